@@ -179,6 +179,11 @@ typedef struct {
     int32_t candidates;         /* candidates per query kept for the exact re-rank */
     int32_t splits;             /* reference splits (CTAs sharing one query tile) */
     int64_t chunk;              /* references per split */
+                                /* float32 Euclidean searches with k_blocks > 0 run a
+                                   tensor-core filter on pairs of bf16 words first, and the
+                                   fields from k_blocks to list_capacity are that filter's;
+                                   splits and chunk are the select's, which takes the
+                                   queries the filter cannot certify */
     int32_t k_blocks;           /* tensor cores: 128-byte K blocks per operand row */
     int32_t stages;             /* tensor cores: depth of the reference stage ring */
     int32_t whole_tile_stages;  /* tensor cores: 1 when a stage holds a whole reference tile */

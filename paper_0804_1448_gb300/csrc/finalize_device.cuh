@@ -428,7 +428,10 @@ __device__ void gather_cand(const FinalizeArgs& a, int64_t q, WarpScratch& w, in
 // The score of a hit-list key: its high word, a code in [0, 0xffff] that
 // falls linearly with the low-precision score, as a float (exact: the code
 // sits in the mantissa of 2^23 + code).
+// PAIR (operand pairs): -acc, from a high word of 0x7f800000 minus acc's bits.
+template <bool PAIR>
 __device__ __forceinline__ float hit_val(uint32_t hi) {
+    if (PAIR) return -__uint_as_float(0x7f800000u - hi);
     return __uint_as_float(0x4B000000u | hi) - 8388608.f;
 }
 
@@ -498,9 +501,11 @@ __device__ __forceinline__ void hit_totals(const FinalizeArgs& a, int64_t q, int
 // pass reads shared memory; the kept indices are compacted in place, each
 // written at or before the position it was read from (MODE 2).  Longer ones
 // are re-read from global memory at every pass (MODE 0).
-template <int METRIC, int NV, int MODE>
+// PAIR: *acc_cut becomes the largest acc among the listed references that
+// were not kept (0 when all were: those not listed have acc < 0).
+template <int METRIC, int NV, int MODE, bool PAIR>
 __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScratch& w, int lane,
-                                int total) {
+                                int total, float* acc_cut) {
     constexpr bool STAGED = MODE != 0;
     const HitLists& hl = a.hits;
     const int S = hl.S, cap = hl.cap, c = hl.c;
@@ -560,11 +565,11 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
         if constexpr (MODE == 1) {
 #pragma unroll
             for (int i = 0; i < kRegHits; ++i)
-                if (i * 32 + lane < total) f(hit_val(hv[i]));
+                if (i * 32 + lane < total) f(hit_val<PAIR>(hv[i]));
         } else if constexpr (MODE == 2) {
-            for (int e = lane; e < total; e += 32) f(hit_val(static_cast<uint32_t>(w.keys[e] >> 32)));
+            for (int e = lane; e < total; e += 32) f(hit_val<PAIR>(static_cast<uint32_t>(w.keys[e] >> 32)));
         } else {
-            visit_global([&](uint64_t key) { f(hit_val(static_cast<uint32_t>(key >> 32))); });
+            visit_global([&](uint64_t key) { f(hit_val<PAIR>(static_cast<uint32_t>(key >> 32))); });
         }
     };
     for_each([&](float v) {
@@ -607,13 +612,16 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
         return bb < cut1 || (bb == cut1 && (b2.inv == 0.f || b2.bin(v) <= cut2));
     };
     int kept = 0;
+    float cut = 0.f;   // -acc of the best reference this lane cut, 0 at most
     if constexpr (MODE == 2) {
         // in place: every lane reads its entry before any lane writes, and a
         // kept entry goes to a position at or before the one it came from
         for (int e0 = 0; e0 < total; e0 += 32) {
             const int e = e0 + lane;
             const uint64_t key = e < total ? w.keys[e] : 0ull;
-            const bool take = e < total && keep(hit_val(static_cast<uint32_t>(key >> 32)));
+            const float v = hit_val<PAIR>(static_cast<uint32_t>(key >> 32));
+            const bool take = e < total && keep(v);
+            if (PAIR && e < total && !take) cut = fminf(cut, v);
             const unsigned bal = __ballot_sync(0xffffffffu, take);
             __syncwarp();
             const int pos = kept + __popc(bal & ((1u << lane) - 1u));
@@ -625,7 +633,9 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
 #pragma unroll
         for (int i = 0; i < kRegHits; ++i) {
             const int e = i * 32 + lane;
-            const bool take = e < total && keep(hit_val(hv[i]));
+            const float v = hit_val<PAIR>(hv[i]);
+            const bool take = e < total && keep(v);
+            if (PAIR && e < total && !take) cut = fminf(cut, v);
             const unsigned bal = __ballot_sync(0xffffffffu, take);
             const int pos = kept + __popc(bal & ((1u << lane) - 1u));
             if (take && pos < P) w.keys[pos] = static_cast<uint32_t>(w.stage[e]);
@@ -635,9 +645,12 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
         if (lane == 0) w.hist[kBins] = 0;
         __syncwarp();
         visit_global([&](uint64_t key) {
-            if (keep(hit_val(static_cast<uint32_t>(key >> 32)))) {
+            const float v = hit_val<PAIR>(static_cast<uint32_t>(key >> 32));
+            if (keep(v)) {
                 const int pos = atomicAdd(&w.hist[kBins], 1);
                 if (pos < P) w.keys[pos] = key_idx(key);
+            } else if (PAIR) {
+                cut = fminf(cut, v);
             }
         });
         __syncwarp();
@@ -645,6 +658,10 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
     }
     __syncwarp();
     if (kept > P) return -3;
+    if (PAIR) {
+        for (int o = 16; o > 0; o >>= 1) cut = fminf(cut, __shfl_xor_sync(0xffffffffu, cut, o));
+        *acc_cut = -cut;
+    }
     exact_keys<METRIC, NV>(w.keys, kept, a.R, a.d, w.qrow, lane);
     return kept;
 }
@@ -678,6 +695,7 @@ __device__ __forceinline__ void cswap(uint64_t& a, uint64_t& b) {
 __device__ __forceinline__ void queue_fallback(const FinalizeArgs& a, int64_t q, int reason) {
     const int pos = atomicAdd(a.fallback_count, 1);
     a.fallback_list[pos] = static_cast<int32_t>(q);
+    if (a.leave) return;
     if (a.fallback_total) atomicAdd(a.fallback_total, 1ull);
     if (a.fallback_reason) atomicAdd(&a.fallback_reason[reason], 1ull);
 }
@@ -685,9 +703,12 @@ __device__ __forceinline__ void queue_fallback(const FinalizeArgs& a, int64_t q,
 // Query q, start to end, by one warp (lane = its lane): scratch is the warp's
 // shared memory (warp_scratch_bytes for these P, S, d and staging entries).
 // Every step is warp-synchronous; nothing waits on the rest of the CTA.
-template <int METRIC, int NV>
+// crow: the query's row of the candidate set (q unless the pass runs over a
+// queue).  PAIR: hit lists of an operand-pair filter, whose answers are
+// certified by the list's bound.
+template <int METRIC, int NV, bool PAIR = false>
 __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, int64_t q,
-                               unsigned char* scratch, int lane) {
+                               unsigned char* scratch, int lane, int64_t crow) {
     const int S = a.use_hits ? 1 : a.cand.S;
     const int d = a.d, k = a.k;
     const int Lcap = prefix_cap(P, k);
@@ -714,15 +735,17 @@ __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, 
 
     // 1. candidates with exact float32 keys
     int pool;
+    float acc_cut = 0.f;
     if (!a.use_hits) {
         pool = a.cand.S * a.cand.c;
-        gather_cand<METRIC, NV>(a, q, w, lane);
+        gather_cand<METRIC, NV>(a, crow, w, lane);
     } else {
         if (over) pool = -2;
         else if (total < a.hits.c && total < a.m) pool = -1;
-        else if (total <= kStage) pool = gather_hits_impl<METRIC, NV, 1>(a, q, P, w, lane, total);
-        else if (total <= stage_all) pool = gather_hits_impl<METRIC, NV, 2>(a, q, P, w, lane, total);
-        else pool = gather_hits_impl<METRIC, NV, 0>(a, q, P, w, lane, total);
+        else if (total <= kStage) pool = gather_hits_impl<METRIC, NV, 1, PAIR>(a, q, P, w, lane, total, &acc_cut);
+        else if (total <= stage_all)
+            pool = gather_hits_impl<METRIC, NV, 2, PAIR>(a, q, P, w, lane, total, &acc_cut);
+        else pool = gather_hits_impl<METRIC, NV, 0, PAIR>(a, q, P, w, lane, total, &acc_cut);
         if (pool < 0) {
             if (lane == 0) queue_fallback(a, q, -pool - 1);
             return;
@@ -897,8 +920,23 @@ __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, 
     };
     auto source_of = [&](int s) { return (w.runs[s] >= 0) ? w.perm[s] : s; };
 
-    // 4. completeness of a float32 candidate set: the references left out by a
-    //    split have keys >= that split's largest kept key
+    // the k-th distance, rounded up by its error
+    auto kth_upper = [&]() {
+        const int sk = source_of(kk - 1);
+        return (w.runs[kk - 1] >= 0) ? static_cast<double>(refined(w.d64[sk])) * (1.0 + 1e-6)
+                                     : static_cast<double>(key_dist(w.sorted[sk])) * (1.0 + a.rel);
+    };
+    // 4. completeness.  Operand pairs: the references that were not kept have
+    //    acc <= acc_cut, so they are at least bound - 2 acc_cut away
+    if (PAIR) {
+        const double lower = static_cast<double>(a.hits.bound[q]) - 2.0 * static_cast<double>(acc_cut);
+        if (kk < k || !(lower > kth_upper())) {
+            if (lane == 0) queue_fallback(a, q, 3);
+            return;
+        }
+    }
+    //    A float32 candidate set: the references left out by a split have
+    //    keys >= that split's largest kept key
     if (!a.use_hits && a.cand.exact && kk > 0) {
         const double rel = a.rel;
         const CandidateSet& cs = a.cand;
@@ -914,11 +952,7 @@ __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, 
             }
         }
         if (have) {
-            const int sk = source_of(kk - 1);
-            const double upper = (w.runs[kk - 1] >= 0)
-                                     ? static_cast<double>(refined(w.d64[sk])) * (1.0 + 1e-6)
-                                     : static_cast<double>(key_dist(w.sorted[sk])) * (1.0 + rel);
-            if (!(lower > upper) || kk < k) {
+            if (!(lower > kth_upper()) || kk < k) {
                 if (lane == 0) queue_fallback(a, q, 3);
                 return;
             }
@@ -945,19 +979,29 @@ __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, 
     }
 }
 
-template <int METRIC, int NV>
+template <int METRIC, int NV, bool PAIR>
 __global__ void __launch_bounds__(kFinThreads, 4)
 finalize_kernel(FinalizeArgs a, int P, int warps_per_block, int stage_entries) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int64_t q = static_cast<int64_t>(blockIdx.x) * warps_per_block + warp;
+    const int64_t row = static_cast<int64_t>(blockIdx.x) * warps_per_block + warp;
+    int64_t q = row;
     if (a.fb_done && blockIdx.x == 0 && static_cast<int>(threadIdx.x) < a.fb_slots)
         a.fb_done[threadIdx.x] = 0;   // the fallback's chunk counters, for this search
     if (q >= a.n) return;   // warp-uniform: no block-level sync below
+    if (!PAIR && a.from.list) {
+        const int count = *a.from.count;
+        if (row >= count) return;
+        q = a.from.list[row];
+        if (count <= kDirectQueue) {   // too few for the select: no candidates to finish
+            if (lane == 0) queue_fallback(a, q, 3);
+            return;
+        }
+    }
     const int S = a.use_hits ? 1 : a.cand.S;
     const size_t per_warp =
         warp_scratch_bytes(P, prefix_cap(P, a.k), S, a.d, a.use_hits ? stage_entries : 0);
-    finalize_query<METRIC, NV>(a, P, stage_entries, q, smem_raw + per_warp * warp, lane);
+    finalize_query<METRIC, NV, PAIR>(a, P, stage_entries, q, smem_raw + per_warp * warp, lane, row);
 }
 
 // ---------------------------------------------------------------------------

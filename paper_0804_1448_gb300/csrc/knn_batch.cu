@@ -142,7 +142,7 @@ __device__ __noinline__ void final_rows(const FinalizeArgs& fa, const BatchInst&
     if (warp >= I.fin_wq) return;
     unsigned char* scratch = smem + static_cast<size_t>(I.fin_pw) * warp;
     for (int64_t q = q0 + warp; q < q1; q += I.fin_wq)
-        finalize_query<kL2, NV>(fa, I.fin_P, I.fin_se, q, scratch, lane);
+        finalize_query<kL2, NV>(fa, I.fin_P, I.fin_se, q, scratch, lane, q);
 }
 
 // Rows [r0, r1) of R (REF) or Q into the instance's augmented low-precision

@@ -20,12 +20,17 @@ using namespace knn;
 
 namespace {
 
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 10;
 // A host-buffer search runs in up to kMaxParts parts of at least
 // kPartMinQueries queries each (four parts measured no faster than two at
 // n = 38400: 62.2 against 62.3-62.4 million queries/s end to end).
 constexpr int kMaxParts = 2;
 constexpr int64_t kPartMinQueries = 4096;
+
+// The most workspace a search may plan for its operand-pair filter.  Ten
+// million queries against 5000 references would hold 41 GB of hit lists for
+// what the select does in 3; a set of four million, d = 128, needs 3 GB.
+constexpr size_t kPairMaxBytes = 16ull << 30;
 
 // Device counters owned by a handle.
 struct Counters {
@@ -304,6 +309,10 @@ void stage(knn_ctx* h, cudaStream_t st, const char* name) {
 struct SearchPlan {
     bool tensor = false;
     bool small = false;      // float32: all m distances per query in shared memory (knn_small.cu)
+    // float32, Euclidean: the filter on operand pairs runs first (plan, kp and
+    // the tensor-core slices below are its own); S, chunk and c stay those of
+    // the CUDA-core select, which takes the queries the filter cannot certify
+    bool pair = false;
     int c_need = 0;          // small: the nearest keys a query must keep (c slots, c >= c_need)
     int prec = 0;
     int kp = 0;
@@ -313,15 +322,34 @@ struct SearchPlan {
     TcPlan plan{};
     int64_t fb_grid = 1;
     size_t off_cand = 0, off_ql = 0, off_gmax = 0, off_lists = 0, off_counts = 0, off_qs = 0;
+    size_t off_rl = 0, off_queue = 0;   // operand pairs: reference copy; queued queries and their count
     size_t off_list = 0, off_scr = 0, off_fbdone = 0, off_q = 0, off_dist = 0, off_idx = 0;
     size_t bytes = 0;
 };
+
+// The operand-pair filter of a float32 Euclidean search (c candidates), when
+// its rows fit the tensor-core tile (d up to 187) and its pilot runs.  It is
+// the faster form at every size above the small-set select's: one query among
+// 5000 references, d = 8, 52 us against 97 us with the CUDA-core select; 64
+// among 2 million, d = 96, 0.80 ms against 1.96; 4000 among 100000, d = 128,
+// 0.44 ms against 3.90; n = m = 38400, d = 96, 1.08 ms against 8.57.
+bool plan_pair(int64_t n, int64_t m, int32_t d, int32_t c, int sm_share, SearchPlan* p) {
+    if (!pair_rows_fit(d) || 2 * c + 32 > finalize_max_pool()) return false;
+    const int kp = tc_padded_dim(d, kPair);
+    const TcPlan t = tc_plan(n, pair_tiles(m) * kPairTile, d, kp, kPair, c, sm_share);
+    if (t.stages == 0 || !t.raw || !t.pilot) return false;
+    p->plan = t;
+    p->plan.m_set = m;
+    p->prec = kPair;
+    p->kp = kp;
+    return true;
+}
 
 // sm_share: how many SMs the search should fill on its own (all of them for a
 // lone search; fewer when several run side by side in a batch).
 knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision, int64_t n, int32_t k,
                           knn_metric metric, int io_on_device, int sm_share, SearchPlan* sp,
-                          int64_t fb_cap_bytes = 64LL << 20) {
+                          int64_t fb_cap_bytes = 64LL << 20, bool allow_pair = true) {
     SearchPlan p;
     p.tensor = (metric == KNN_L2) && precision != KNN_FP32;
     p.prec = p.tensor ? (precision == KNN_BF16 ? kBF16 : kTF32) : 0;
@@ -358,7 +386,7 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
         if (p.plan.stages == 0 ||
             (small_select_fits(m, d) && (!p.plan.pilot || small_share < kSmallSelectShare)))
             return plan_search_md(h, m, d, KNN_FP32, n, k, metric, io_on_device, sm_share, sp,
-                                  fb_cap_bytes);
+                                  fb_cap_bytes, allow_pair);
         p.S = p.plan.S;
         p.chunk = p.plan.chunk;
     } else if (small_select_fits(m, d)) {
@@ -373,6 +401,7 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
         if (static_cast<int64_t>(S) * p.c > finalize_max_pool()) return KNN_ERR_UNSUPPORTED;
         p.S = S;
         p.chunk = chunk;
+        p.pair = allow_pair && metric == KNN_L2 && plan_pair(n, m, d, p.c, sm_share, &p);
     }
 
     // fallback grid: scratch of grid * m doubles, at most fb_cap_bytes
@@ -382,13 +411,22 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
 
     // workspace layout
     Carve cv;
-    if (p.tensor) {
-        const size_t elt = (p.prec == kBF16) ? 2 : 4;
+    if (p.pair) {
+        p.off_rl = cv.take(static_cast<size_t>(pair_tiles(m)) * kPairTile * p.kp * 2);
+        p.off_queue = cv.take((static_cast<size_t>(n) + 1) * sizeof(int32_t));
+    }
+    if (p.tensor || p.pair) {
+        const size_t elt = p.prec == kTF32 ? 4 : 2;
         p.off_ql = cv.take(static_cast<size_t>(n) * p.kp * elt);
         if (p.plan.pilot) p.off_gmax = cv.take(static_cast<size_t>(n) * p.plan.G * 4);
-        p.off_lists = cv.take(static_cast<size_t>(n) * p.S * p.plan.groups * p.plan.cap *
-                              sizeof(uint64_t));
-        p.off_counts = cv.take(static_cast<size_t>(n) * p.S * p.plan.groups * sizeof(int32_t));
+        size_t list_bytes = static_cast<size_t>(n) * p.plan.S * p.plan.groups * p.plan.cap *
+                            sizeof(uint64_t);
+        if (p.pair) {   // the lists are consumed before the select writes its candidates
+            list_bytes = std::max(list_bytes, static_cast<size_t>(n) * p.S * p.c * sizeof(uint64_t));
+        }
+        p.off_lists = cv.take(list_bytes);
+        p.off_cand = p.off_lists;
+        p.off_counts = cv.take(static_cast<size_t>(n) * p.plan.S * p.plan.groups * sizeof(int32_t));
         p.off_qs = cv.take(static_cast<size_t>(n) * sizeof(float));
     } else {
         p.off_cand = cv.take(static_cast<size_t>(n) * p.S * p.c * sizeof(uint64_t));
@@ -402,14 +440,41 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
         p.off_idx = cv.take(static_cast<size_t>(n) * k * sizeof(int32_t));
     }
     p.bytes = cv.off;
+    // the filter's copies and lists are scratch the select alone does not need:
+    // it runs alone where they would pass the handle's limit, or kPairMaxBytes
+    const size_t most = h->opt.workspace_limit > 0
+                            ? std::min(kPairMaxBytes, static_cast<size_t>(h->opt.workspace_limit))
+                            : kPairMaxBytes;
+    if (p.pair && p.bytes > most)
+        return plan_search_md(h, m, d, precision, n, k, metric, io_on_device, sm_share, sp,
+                              fb_cap_bytes, false);
     *sp = p;
     return KNN_OK;
 }
 
 knn_status plan_search(const knn_ctx* h, int64_t n, int32_t k, knn_metric metric, int io_on_device,
-                       SearchPlan* sp) {
+                       SearchPlan* sp, bool allow_pair = true) {
     return plan_search_md(h, h->ref->m, h->ref->d, h->opt.precision, n, k, metric, io_on_device,
-                          h->num_sms, sp);
+                          h->num_sms, sp, 64LL << 20, allow_pair);
+}
+
+// Plan a search on st and hold its workspace, `extra` bytes after the plan's
+// own included.  A float32 search whose operand-pair scratch cannot be had --
+// no memory, or a capturing stream and a workspace that would have to grow --
+// runs the select alone, which needs less.
+knn_status plan_and_hold(knn_ctx* h, int64_t n, int32_t k, knn_metric metric, int io_on_device,
+                         cudaStream_t st, size_t extra, SearchPlan* sp) {
+    knn_status s = plan_search(h, n, k, metric, io_on_device, sp);
+    if (s != KNN_OK) return s;
+    if (sp->pair && sp->bytes + extra > h->ws_bytes) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        KNN_CUDA(h, cudaStreamIsCapturing(st, &cap));
+        s = cap == cudaStreamCaptureStatusNone ? ensure_workspace(h, sp->bytes + extra) : KNN_ERR_OOM;
+        if (s != KNN_ERR_OOM) return s;
+        s = plan_search(h, n, k, metric, io_on_device, sp, false);
+        if (s != KNN_OK) return s;
+    }
+    return ensure_workspace(h, sp->bytes + extra);
 }
 
 // The reference data one search reads: a handle's reference set, or the
@@ -439,11 +504,20 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
     auto mark = [&](const char* name) {
         if (stages) stage(h, st, name);
     };
-    KNN_CUDA(h, cudaMemsetAsync(fallback_count, 0, sizeof(int32_t), st));
     FinalizeArgs fa{};
-    if (sp.tensor) {
+    QueryQueue queue{};
+    if (sp.pair) {
+        queue.count = reinterpret_cast<int32_t*>(ws + sp.off_queue);
+        queue.list = queue.count + 1;
+    } else {
+        KNN_CUDA(h, cudaMemsetAsync(fallback_count, 0, sizeof(int32_t), st));
+    }
+    if (sp.tensor || sp.pair) {
         const TcPlan& plan = sp.plan;
         const int prec = sp.prec;
+        const void* R_lp = sp.pair ? ws + sp.off_rl : rv.R_lp;
+        const int32_t kp = sp.pair ? sp.kp : rv.kp;
+        const int64_t mt = sp.pair ? plan.tiles * kPairTile : m;
         void* Ql = ws + sp.off_ql;
         uint64_t* lists = reinterpret_cast<uint64_t*>(ws + sp.off_lists);
         int32_t* counts = reinterpret_cast<int32_t*>(ws + sp.off_counts);
@@ -452,27 +526,31 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
         qs.qscale = reinterpret_cast<float*>(ws + sp.off_qs);
         HitScale qs_prep = qs;   // the threshold pass sets B when there is one
         if (plan.pilot) qs_prep.qscale = nullptr;
-        KNN_CUDA(h, launch_prepare_query(Qd, n, d, rv.kp, prec, Ql, qs_prep, Q_copy, st, l));
+        if (sp.pair)
+            KNN_CUDA(h, launch_prepare_pair(rv.R, m, Qd, n, d, kp, ws + sp.off_rl, Ql, qs.qscale,
+                                            queue.count, fallback_count, st, l));
+        else
+            KNN_CUDA(h, launch_prepare_query(Qd, n, d, kp, prec, Ql, qs_prep, Q_copy, st, l));
         if (Q_copy) Qd = Q_copy;
         mark("prepare_q");
         if (prep_done) KNN_CUDA(h, cudaEventRecord(prep_done, st));
         if (plan.pilot) {
             uint32_t* gmax = reinterpret_cast<uint32_t*>(ws + sp.off_gmax);
-            KNN_CUDA(h, launch_tc_pilot(plan, Ql, n, rv.R_lp, m, rv.kp, prec, gmax, &ctr->error_flag,
-                                        st, l));
+            KNN_CUDA(h, launch_tc_pilot(plan, Ql, n, R_lp, mt, kp, prec, gmax, &ctr->error_flag, st, l));
             mark("tc_pilot");
-            KNN_CUDA(h, launch_tc_threshold(plan, gmax, n, d, rv.kp, prec, Ql, qs, st, l));
+            KNN_CUDA(h, launch_tc_threshold(plan, gmax, n, d, kp, prec, Ql, qs, st, l));
             mark("tc_threshold");
         }
-        KNN_CUDA(h, launch_tc_filter(plan, Ql, n, rv.R_lp, m, rv.kp, prec, lists, counts, qs.qscale,
+        KNN_CUDA(h, launch_tc_filter(plan, Ql, n, R_lp, mt, kp, prec, lists, counts, qs.qscale,
                                      &ctr->error_flag, st, l));
         mark("tc_filter");
         fa.use_hits = 1;
         fa.hits.keys = lists;
         fa.hits.counts = counts;
-        fa.hits.S = plan.groups * S;   // one list per (split, epilogue column group)
+        fa.hits.S = plan.groups * plan.S;   // one list per (split, epilogue column group)
         fa.hits.cap = plan.cap;
         fa.hits.c = c;
+        fa.hits.bound = sp.pair ? qs.qscale : nullptr;
         fa.cand.exact = 0;
         fa.cand.S = 1;
         fa.cand.c = c;
@@ -510,8 +588,34 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
     fa.fallback_reason = ctr->fallback_reason;
     fa.fb_done = reinterpret_cast<int32_t*>(ws + sp.off_fbdone);
     fa.fb_slots = static_cast<int32_t>(sp.fb_grid);
-    KNN_CUDA(h, launch_finalize(fa, st, l));
-    mark("finalize");
+    if (sp.pair) {
+        // the filter's answers; the queries it cannot certify go through the
+        // CUDA-core select (a few: straight to the exact fallback)
+        FinalizeArgs fp = fa;
+        fp.fallback_count = queue.count;
+        fp.fallback_list = queue.list;
+        fp.leave = 1;
+        fp.fb_done = nullptr;
+        KNN_CUDA(h, launch_finalize(fp, st, l));
+        mark("finalize");
+        CandidateSet cs;
+        cs.keys = reinterpret_cast<uint64_t*>(ws + sp.off_cand);
+        cs.n = n;
+        cs.S = S;
+        cs.c = c;
+        cs.chunk = sp.chunk;
+        cs.exact = 1;
+        KNN_CUDA(h, launch_cc_select(Qd, n, rv.R, m, d, metric, cs, st, l, queue));
+        fa.use_hits = 0;
+        fa.hits = HitLists{};
+        fa.cand = cs;
+        fa.from = queue;
+        KNN_CUDA(h, launch_finalize(fa, st, l));
+        mark("cc_queued");
+    } else {
+        KNN_CUDA(h, launch_finalize(fa, st, l));
+        mark("finalize");
+    }
     KNN_CUDA(h, launch_fallback(fa, reinterpret_cast<double*>(ws + sp.off_scr),
                                 static_cast<int32_t>(sp.fb_grid), fa.fb_done, st, l));
     mark("fallback");
@@ -593,7 +697,7 @@ knn_status plan_batch(const knn_ctx* h, const knn_instance* inst, int32_t count,
         SearchPlan& sp = bp->sp[i];
         knn_status s = plan_search_md(h, x.m, x.d, h->opt.precision, x.n, x.k,
                                       static_cast<knn_metric>(x.metric), 1, sm_share, &sp,
-                                      4LL << 20);
+                                      4LL << 20, false);   // no reference copy per instance
         if (s != KNN_OK) return s;
         bp->base[i] = cv.take(sp.bytes);
         bp->fbc[i] = cv.take(sizeof(int32_t));
@@ -1053,7 +1157,7 @@ knn_status knn_search(knn_handle h, const float* Q, int64_t n, int32_t d, int32_
     const int64_t m = rs.m;
 
     SearchPlan sp;
-    knn_status s = plan_search(h, n, k, metric, io_on_device, &sp);
+    knn_status s = plan_and_hold(h, n, k, metric, io_on_device, st, 0, &sp);
     if (s != KNN_OK) return s;
     if (sp.tensor) {
         s = build_lowp_on(h, refp, sp.prec);
@@ -1067,8 +1171,6 @@ knn_status knn_search(knn_handle h, const float* Q, int64_t n, int32_t d, int32_
         KNN_CUDA(h, cudaMalloc(&h->qw, static_cast<size_t>(n) * d * sizeof(float)));
         h->qw_bytes = static_cast<size_t>(n) * d * sizeof(float);
     }
-    s = ensure_workspace(h, sp.bytes);
-    if (s != KNN_OK) return s;
     unsigned char* ws = h->ws;
 
     const float* Qd = Q;
@@ -1365,19 +1467,20 @@ knn_status knn_search_self(knn_handle h, int32_t k, knn_metric metric, float* di
     RefSet& rs = *h->ref;
     const int64_t n = rs.m;
     SearchPlan sp;
-    s = plan_search(h, n, k + 1, metric, 1, &sp);
+    // the (k+1)-neighbour rows go to workspace after the search's own slices
+    Carve rows;
+    rows.take(static_cast<size_t>(n) * (k + 1) * sizeof(float));
+    rows.take(static_cast<size_t>(n) * (k + 1) * sizeof(int32_t));
+    s = plan_and_hold(h, n, k + 1, metric, 1, st, rows.off, &sp);
     if (s != KNN_OK) return s;
     if (sp.tensor) {
         s = build_lowp(h, sp.prec);
         if (s != KNN_OK) return s;
     }
-    // the (k+1)-neighbour rows go to workspace after the search's own slices
     Carve cv;
     cv.off = sp.bytes;
     const size_t off_d = cv.take(static_cast<size_t>(n) * (k + 1) * sizeof(float));
     const size_t off_i = cv.take(static_cast<size_t>(n) * (k + 1) * sizeof(int32_t));
-    s = ensure_workspace(h, cv.off);
-    if (s != KNN_OK) return s;
     unsigned char* ws = h->ws;
     float* dtmp = reinterpret_cast<float*>(ws + off_d);
     int32_t* itmp = reinterpret_cast<int32_t*>(ws + off_i);
@@ -1428,7 +1531,7 @@ knn_status knn_explain_plan(int64_t n, int64_t m, int32_t d, int32_t k, knn_metr
     o.candidates = sp.c;
     o.splits = sp.S;
     o.chunk = sp.chunk;
-    if (sp.tensor) {
+    if (sp.tensor || sp.pair) {
         o.k_blocks = sp.plan.kb;
         o.stages = sp.plan.stages;
         o.whole_tile_stages = sp.plan.kbs == sp.plan.kb ? 1 : 0;

@@ -145,10 +145,17 @@ __device__ __forceinline__ float pair_hi(uint64_t v) { return __uint_as_float(st
 // Euclidean products run as two-lane float32 fused multiply-adds; the
 // threads below kTM (below ROWS, in a CTA's first tile) also sum the squares
 // of reference (query) tid's staged coordinates, its squared norm.
-template <int METRIC, int ROWS>
+// QUEUED: the CTA's queries are those of a queue (nothing to do while it is no
+// longer than kDirectQueue), candidate row i being that of the queue's i-th.
+template <int METRIC, int ROWS, bool QUEUED>
 __global__ void __launch_bounds__(kThreads, CCShape<ROWS>::MINB)
 cc_select_kernel(const float* __restrict__ Q, int64_t n, const float* __restrict__ R,
-                 int64_t m, int32_t d, CandidateSet cand) {
+                 int64_t m, int32_t d, CandidateSet cand, QueryQueue from) {
+    if constexpr (QUEUED) {
+        const int count = *from.count;
+        if (count <= kDirectQueue || static_cast<int64_t>(blockIdx.x) * ROWS >= count) return;
+        n = count;
+    }
     using S = CCShape<ROWS>;
     static_assert(S::TY * S::TX == kThreads, "thread shape");
     static_assert(S::TY * S::RR == ROWS && S::TX * S::CN == kTM, "tile shape");
@@ -221,7 +228,7 @@ cc_select_kernel(const float* __restrict__ Q, int64_t n, const float* __restrict
             const int e = tid + u * kThreads, r = e / kDK, t = e % kDK;
             const int64_t gq = qbase + r;
             const int gt = dbase + t;
-            pq[u] = (gq < n && gt < d) ? Q[gq * d + gt] : 0.f;
+            pq[u] = (gq < n && gt < d) ? Q[(QUEUED ? from.list[gq] : gq) * d + gt] : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < RPT; ++u) {
@@ -421,15 +428,16 @@ cc_select_kernel(const float* __restrict__ Q, int64_t n, const float* __restrict
     }
 }
 
-template <int METRIC, int ROWS>
+template <int METRIC, int ROWS, bool QUEUED = false>
 cudaError_t launch_rows(const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
-                        const CandidateSet& cand, cudaStream_t st) {
-    auto kern = cc_select_kernel<METRIC, ROWS>;
+                        const CandidateSet& cand, cudaStream_t st,
+                        const QueryQueue& from = QueryQueue{}) {
+    auto kern = cc_select_kernel<METRIC, ROWS, QUEUED>;
     const size_t smem = cc_smem_bytes<ROWS>(cand.c);
-    cudaError_t err = allow_smem<cc_select_kernel<METRIC, ROWS>>(smem);
+    cudaError_t err = allow_smem<cc_select_kernel<METRIC, ROWS, QUEUED>>(smem);
     if (err != cudaSuccess) return err;
     dim3 grid(static_cast<unsigned>((n + ROWS - 1) / ROWS), static_cast<unsigned>(cand.S));
-    kern<<<grid, kThreads, smem, st>>>(Q, n, R, m, d, cand);
+    kern<<<grid, kThreads, smem, st>>>(Q, n, R, m, d, cand, from);
     return cudaGetLastError();
 }
 
@@ -510,11 +518,17 @@ int cc_max_candidates() {
 
 cudaError_t launch_cc_select(const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
                              int32_t metric, const CandidateSet& cand, cudaStream_t st,
-                             int* launches) {
+                             int* launches, const QueryQueue& from) {
     int64_t per_sm = 1;
     const int rows = cc_rows(n, cand.c, &per_sm);
     if (rows == 16 && cc_smem_bytes<16>(cand.c) > kSmemCap) return cudaErrorInvalidValue;
     if (launches) ++*launches;
+    if (from.list) {
+        if (metric != kL2) return cudaErrorInvalidValue;
+        return rows == 128 ? launch_rows<kL2, 128, true>(Q, n, R, m, d, cand, st, from)
+               : rows == 64 ? launch_rows<kL2, 64, true>(Q, n, R, m, d, cand, st, from)
+                            : launch_rows<kL2, 16, true>(Q, n, R, m, d, cand, st, from);
+    }
     if (metric == kL2)
         return rows == 128 ? launch_rows<kL2, 128>(Q, n, R, m, d, cand, st)
                : rows == 64 ? launch_rows<kL2, 64>(Q, n, R, m, d, cand, st)

@@ -9,6 +9,9 @@
 //                  form (knn_cc.cu) computes float32 distances from coordinate
 //                  differences; the tensor-core form (knn_tc.cu) computes the
 //                  cross term q.r with tcgen05 and ranks by ||r||^2 - 2 q.r.
+//                  A float32 Euclidean search takes the tensor-core form on
+//                  pairs of bf16 words, whose answers the finalize certifies;
+//                  the queries it cannot certify take the CUDA-core form.
 //   2. finalize -- per query: exact float32 distances of the candidates, a sort
 //                  by (distance, index), a float64 re-check of candidates whose
 //                  float32 distances are within rounding of each other, and the
@@ -107,7 +110,19 @@ struct HitLists {
     int32_t S;
     int32_t cap;
     int32_t c;              // keep (at least) the best c before the exact re-rank
+    const float* bound;     // operand pairs: [n], every reference is at least bound - 2 acc
+                            // away (squared), and the keys' high word is 0x7f800000 minus
+                            // the bits of acc, 0 for a reference not listed; else null
 };
+
+// The queries one pass left to the next: list[0 .. *count).  A pass over a
+// queue does nothing while it holds kDirectQueue queries or fewer: those go
+// straight to the exact fallback, which spreads each over the GPU.
+struct QueryQueue {
+    int32_t* list;    // null: the pass covers every query
+    int32_t* count;
+};
+constexpr int kDirectQueue = 32;
 
 struct FinalizeArgs {
     int32_t use_hits;       // 0: candidates come from `cand`; 1: from `hits`
@@ -122,6 +137,10 @@ struct FinalizeArgs {
     int32_t* idx_out;
     int32_t* fallback_count;   // device counter of queued queries
     int32_t* fallback_list;    // [n] query ids
+    QueryQueue from;           // list: only these queries, candidate row i being that of
+                               // the queue's i-th; null: all n
+    int32_t leave;             // 1: fallback_list is the next pass's queue, not the exact
+                               // fallback's (its queries are not counted as such)
     unsigned long long* recheck_counter;
     unsigned long long* fallback_total;
     unsigned long long* fallback_reason;   // [4]: short list, overflow, wide cut, uncertified
@@ -137,9 +156,11 @@ struct FinalizeArgs {
 // ---- launchers (return cudaSuccess or the launch error) -------------------
 
 // CUDA-core fused distance + top-c.  Writes cand (exact = 1).
+// from.list: only the queue's queries (Euclidean), candidate row i being that
+// of its i-th.
 cudaError_t launch_cc_select(const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
                              int32_t metric, const CandidateSet& cand, cudaStream_t st,
-                             int* launches);
+                             int* launches, const QueryQueue& from = QueryQueue{});
 
 // The largest c launch_cc_select supports.
 int cc_max_candidates();
@@ -198,7 +219,8 @@ cudaError_t launch_fallback(const FinalizeArgs& a, double* scratch, int32_t slot
 
 // ---- tensor-core path (knn_tc.cu) -----------------------------------------
 
-enum LowPrecision : int { kTF32 = 1, kBF16 = 2 };
+// kPair: float32 rows as pairs of bf16 words (the float32 search's own filter).
+enum LowPrecision : int { kTF32 = 1, kBF16 = 2, kPair = 3 };
 
 // Row length (elements) of the low-precision operand copies: d coordinates,
 // four augmentation words (norm halves, threshold halves), zero padded to a
@@ -224,6 +246,9 @@ struct TcPlan {
     int32_t pilot;       // 0: no pilot, every reference is appended
     int32_t cap;         // list capacity per (query, split, column group)
     int32_t raw;         // filter stages hit values as float32 (else 16-bit codes)
+    int32_t hs;          // operand pairs: K steps of the upper words
+    int64_t tiles;       // operand pairs: reference tiles of the set
+    int64_t m_set;       // operand pairs: references of the set
     size_t smem_filter;
 };
 // smem_limit: the dynamic shared memory an item may use (the persistent batch
@@ -241,6 +266,16 @@ struct HitScale {
     const uint32_t* rmax2;
     float* qscale;   // [n]
 };
+
+// Operand pairs (rows of up to kPairMaxD coordinates): both copies of a search
+// in one launch, the queries' squared norms, and its two queue counters
+// cleared.  R_lp holds whole tiles, pair_tiles(m) of them.
+constexpr int64_t kPairTile = 256;
+inline int64_t pair_tiles(int64_t m) { return (m + kPairTile - 1) / kPairTile; }
+bool pair_rows_fit(int32_t d);
+cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* Q, int64_t n, int32_t d,
+                                int32_t kp, void* R_lp, void* Q_lp, float* qnorm, int32_t* count0,
+                                int32_t* count1, cudaStream_t st, int* launches);
 
 // Reference copy [r, -||r||^2/2 (hi, lo), 1, 1, 0..], float32 norms and their maximum.
 cudaError_t launch_prepare_ref(const float* R, int64_t m, int32_t d, int32_t kp, int prec,

@@ -36,7 +36,7 @@ bool tc_make_map(CUtensorMap* map, const void* base, int64_t rows, int kp, int p
                  int box_kb) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const int elt = (prec == kBF16) ? 2 : 4;
+    const int elt = (prec == kTF32) ? 4 : 2;
     const int kb = kp * elt / kAtomBytes;
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(kAtomBytes / elt), static_cast<cuuint64_t>(rows),
                           static_cast<cuuint64_t>(kb)};
@@ -45,7 +45,7 @@ bool tc_make_map(CUtensorMap* map, const void* base, int64_t rows, int kp, int p
                          static_cast<cuuint32_t>(box_kb > 0 ? box_kb : kb)};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = fn(map,
-                    prec == kBF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                    prec == kTF32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
                     3, const_cast<void*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -103,6 +103,9 @@ template <bool PILOT>
 cudaError_t dispatch(const TcPlan& p, int prec, const CUtensorMap& mq, const CUtensorMap& mr,
                      const TcArgs& a, cudaStream_t st) {
     if (prec == kBF16) return dispatch_kb<kBF16, PILOT>(p, mq, mr, a, st);
+    // operand pairs always stage raw values behind a pilot, and their MMA
+    // issue has run-time step counts
+    if (prec == kPair) return launch_kernel<kPair, PILOT, 0, PILOT ? 0 : 1>(p, mq, mr, a, st);
     return dispatch_kb<kTF32, PILOT>(p, mq, mr, a, st);
 }
 
@@ -122,6 +125,9 @@ TcArgs base_args(const TcPlan& p, int64_t n, int64_t m, int32_t* error_flag) {
     a.gps = 32 / p.gsize;
     a.cap = p.cap;
     a.append_all = p.pilot ? 0 : 1;
+    a.hs = p.hs;
+    a.rank_stride = static_cast<int32_t>(p.tiles);
+    a.m_set = static_cast<uint32_t>(p.m_set);
     a.error_flag = error_flag;
     return a;
 }
@@ -144,7 +150,10 @@ cudaError_t launch_wait_probe(int32_t* error_flag, uint64_t limit_ns, cudaStream
     return cudaGetLastError();
 }
 
+bool pair_rows_fit(int32_t d) { return d >= 1 && d <= kPairMaxD; }
+
 int tc_padded_dim(int32_t d, int prec) {
+    if (prec == kPair) return (pair_ksteps(d) + 3) / 4 * 64;
     const int step = (prec == kBF16) ? 64 : 32;   // whole 128-byte K blocks per row
     return (d + kAugCols + step - 1) / step * step;
 }
@@ -153,13 +162,18 @@ TcPlan tc_plan(int64_t n, int64_t m, int32_t d, int32_t kp, int prec, int32_t c,
                size_t smem_limit, int64_t force_chunk) {
     const size_t kSmemLimit = smem_limit;
     TcPlan p{};
-    const int elt = (prec == kBF16) ? 2 : 4;
+    const int elt = (prec == kTF32) ? 4 : 2;
     const int kstep = 32 / elt;                    // elements per MMA K step
     p.mt = 1;
     p.rb = kTileN;
     p.groups = kGroups;
     p.kb = kp * elt / kAtomBytes;
     p.ksteps = (d + kAugCols + kstep - 1) / kstep;
+    if (prec == kPair) {
+        p.ksteps = pair_ksteps(d);
+        p.hs = pair_hsteps(d);
+        p.tiles = m / kTileN;    // the caller passes whole tiles
+    }
     p.stages = 0;
     // whole-tile stages (one TMA box and one wait per tile) when two fit,
     // else single-K-block stages, as many as fit
@@ -180,7 +194,7 @@ TcPlan tc_plan(int64_t n, int64_t m, int32_t d, int32_t kp, int prec, int32_t c,
             if (tc_smem_bytes(p.kb, 1, s, false, true) <= kSmemLimit) s_raw = s;
         if (s_codes > 0) {
             p.kbs = 1;
-            p.raw = (s_raw >= 3 || (s_raw > 0 && s_raw == s_codes)) ? 1 : 0;
+            p.raw = (s_raw >= 3 || (s_raw > 0 && (s_raw == s_codes || prec == kPair))) ? 1 : 0;
             p.stages = p.raw ? s_raw : s_codes;
         }
     }
@@ -305,6 +319,20 @@ cudaError_t launch_prepare_ref(const float* R, int64_t m, int32_t d, int32_t kp,
     return cudaGetLastError();
 }
 
+cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* Q, int64_t n, int32_t d,
+                                int32_t kp, void* R_lp, void* Q_lp, float* qnorm, int32_t* count0,
+                                int32_t* count1, cudaStream_t st, int* launches) {
+    const int64_t tiles = pair_tiles(m);
+    const int64_t ref_warps = tiles * kTileN / kPairRows;
+    const int64_t warps = ref_warps + (n + kPairRows - 1) / kPairRows;
+    const unsigned grid = static_cast<unsigned>((warps * 32 + 255) / 256);
+    prepare_pair_kernel<<<grid, 256, 0, st>>>(R, m, tiles, Q, n, d, kp, static_cast<uint32_t*>(R_lp),
+                                              static_cast<uint32_t*>(Q_lp), qnorm, ref_warps, count0,
+                                              count1);
+    if (launches) ++*launches;
+    return cudaGetLastError();
+}
+
 cudaError_t launch_prepare_query(const float* Q, int64_t n, int32_t d, int32_t kp, int prec,
                                  void* Q_lp, const HitScale& qs, float* Q_copy, cudaStream_t st,
                                  int* launches) {
@@ -363,6 +391,7 @@ cudaError_t launch_tc_threshold(const TcPlan& p, const uint32_t* gmax, int64_t n
                                 cudaStream_t st, int* launches) {
     if (launches) ++*launches;
     if (prec == kBF16) return launch_threshold_p<kBF16>(p, gmax, n, d, kp, Q_lp, qs, st);
+    if (prec == kPair) return launch_threshold_p<kPair>(p, gmax, n, d, kp, Q_lp, qs, st);
     return launch_threshold_p<kTF32>(p, gmax, n, d, kp, Q_lp, qs, st);
 }
 

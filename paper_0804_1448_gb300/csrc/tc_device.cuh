@@ -105,6 +105,10 @@ struct TcArgs {
     int32_t append_all;   // filter: every valid reference passes
     const float* qscale;  // filter: per-query B, a power of two with |acc| < B
     int32_t* error_flag;
+    int32_t hs;           // operand pairs: K steps (16 coordinates) of the upper words
+    int32_t rank_stride;  // operand pairs: reference tiles T (row i*T + g of the set is
+                          // rank i of tile g)
+    uint32_t m_set;       // operand pairs: references of the set (m counts whole tiles)
 };
 
 // A: the query tile, kb K blocks (resident); B: a ring of `stages` stages of
@@ -173,6 +177,21 @@ __device__ __forceinline__ uint32_t packed_bits(uint64_t h) {
     return __float_as_uint(fmaf(lo, 2.f, hi + 8388608.f));
 }
 
+// Operand pairs: the list key of one hit is its acc (>= 0, so its bits rise
+// with it; a negative zero or subnormal counts as 0, and so does a NaN, which
+// can only come from a reference whose distance is not finite): all 32 bits,
+// falling with acc.
+// Rows past the set (j >= m) pass only for a query whose own norm or threshold
+// is not finite; they are never listed.
+__device__ __forceinline__ void append_pair(uint64_t* list, int& cnt, int cap, float x, uint32_t j,
+                                            uint32_t m) {
+    const uint32_t hi = 0x7f800000u - __float_as_uint(fmaxf(x, 0.f));
+    if (j < m) {
+        if (cnt < cap) list[cnt] = (static_cast<uint64_t>(hi) << 32) | j;
+        ++cnt;
+    }
+}
+
 // Position of the highest set bit of x, in 0..31 (31 when x == 0: a valid
 // staging index whose result the caller discards).
 __device__ __forceinline__ uint32_t bfind31(uint32_t x) {
@@ -202,6 +221,28 @@ __device__ __forceinline__ void issue_kblock(uint32_t d_tmem, uint64_t a_desc, u
     for (int ks = 0; ks < 4; ++ks) {
         if (ks < k4)
             mma<PREC>(d_tmem, a_desc + 2 * ks, b_desc + 2 * ks, id, (first && ks == 0) ? 0u : 1u);
+    }
+}
+
+// MMAs of one K block of a tile of operand pairs.  A row holds hs K steps of
+// upper words h, hs of lower words l, and one more step for the norm and
+// threshold words when the padding of the upper ones has no room for them.
+// An upper step of B meets the queries' upper and lower words (h.h + l.h), a
+// lower step their upper words (h.l), the extra step its own: every block of B
+// is loaded once for up to two products, and l.l (2^-16 of the product) is
+// covered by the bound's slack.
+__device__ __forceinline__ void issue_pair_kblock(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                                  int kb, int hs, int nsteps, uint32_t id) {
+    constexpr uint32_t kQStep = kQTileBytes >> 4;
+    auto a_step = [&](int s) { return a_desc + static_cast<uint32_t>(s >> 2) * kQStep + 2u * (s & 3); };
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+        const int s = kb * 4 + ks;
+        if (s < nsteps) {
+            const int sa = (s >= hs && s < 2 * hs) ? s - hs : s;
+            mma<kBF16>(d_tmem, a_step(sa), b_desc + 2 * ks, id, s == 0 ? 0u : 1u);
+            if (s < hs) mma<kBF16>(d_tmem, a_step(hs + s), b_desc + 2 * ks, id, 1u);
+        }
     }
 }
 
@@ -297,7 +338,7 @@ __device__ __forceinline__ void tc_run(const CUtensorMap* tmap_q, const CUtensor
     } else if (warp == 1) {
         // ------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t id = idesc(PREC == kBF16 ? 1 : 2, kBlockM, kTileN);
+            const uint32_t id = idesc(PREC == kTF32 ? 2 : 1, kBlockM, kTileN);
             bool ok = mbar_wait(a_full, 0, abort_flag);
             if (!ok) fail();
             const uint64_t a_desc = sdesc(smem_u32(sA));
@@ -313,7 +354,11 @@ __device__ __forceinline__ void tc_run(const CUtensorMap* tmap_q, const CUtensor
                     if (!mbar_wait(&full[s], (g / NST) & 1, abort_flag)) { fail(); break; }
                     tc_fence_after();
                     const uint64_t b_desc = sdesc(smem_u32(sB + s * stage_bytes));
-                    if (KBT > 0) {
+                    if constexpr (PREC == kPair) {
+                        for (int kb = 0; kb < KB; ++kb)
+                            issue_pair_kblock(d_tmem, a_desc, b_desc + kb * kRStep, kb, a.hs,
+                                              a.ksteps, id);
+                    } else if (KBT > 0) {
 #pragma unroll
                         for (int kb = 0; kb < (KBT > 0 ? KBT : 1); ++kb)
                             issue_kblock<PREC>(d_tmem, a_desc + kb * kQStep, b_desc + kb * kRStep,
@@ -334,9 +379,13 @@ __device__ __forceinline__ void tc_run(const CUtensorMap* tmap_q, const CUtensor
                             break;
                         }
                         tc_fence_after();
-                        issue_kblock<PREC>(d_tmem, a_desc + kb * kQStep,
-                                           sdesc(smem_u32(sB + s * stage_bytes)), a.ksteps - kb * 4,
-                                           kb == 0, id);
+                        if constexpr (PREC == kPair)
+                            issue_pair_kblock(d_tmem, a_desc, sdesc(smem_u32(sB + s * stage_bytes)),
+                                              kb, a.hs, a.ksteps, id);
+                        else
+                            issue_kblock<PREC>(d_tmem, a_desc + kb * kQStep,
+                                               sdesc(smem_u32(sB + s * stage_bytes)),
+                                               a.ksteps - kb * 4, kb == 0, id);
                         tc_commit(&empty[s]);
                     }
                     if (!ok) break;
@@ -363,7 +412,8 @@ __device__ __forceinline__ void tc_run(const CUtensorMap* tmap_q, const CUtensor
         uint32_t* gout = nullptr;
         if (PILOT) gout = a.gmax + q * a.G + static_cast<int64_t>(split) * a.spt * gpt;
         else list = a.lists + ((q * a.S + split) * kGroups + cg) * static_cast<int64_t>(a.cap);
-        const uint32_t off3b = __float_as_uint((!PILOT && active) ? 3.f * a.qscale[q] : 0.f);
+        const uint32_t off3b =
+            __float_as_uint((!PILOT && PREC != kPair && active) ? 3.f * a.qscale[q] : 0.f);
         const uint32_t st_addr = smem_u32(st);
         const uint32_t all_pass = a.append_all ? 0xffffffffu : 0u;
         const uint32_t live = active ? 0xffffffffu : 0u;
@@ -459,6 +509,18 @@ __device__ __forceinline__ void tc_run(const CUtensorMap* tmap_q, const CUtensor
                     const float b3 = __uint_as_float(off3b);
                     const float* stf = reinterpret_cast<const float*>(st) + 31;
                     const uint32_t jb = static_cast<uint32_t>(jt) + 32u * sl + 31u;
+                    // operand pairs: column 64 cg + x of tile g holds row
+                    // (4 x + cg) T + g of the set
+                    const uint32_t pt = PREC == kPair ? 4u * static_cast<uint32_t>(a.rank_stride) : 0u;
+                    const uint32_t pb =
+                        PREC == kPair ? (32u * sl + 31u) * pt +
+                                            static_cast<uint32_t>(cg) * static_cast<uint32_t>(a.rank_stride) +
+                                            static_cast<uint32_t>((jt - cg * kGroupCols) / kTileN)
+                                      : 0u;
+                    auto put_hit = [&](float x, uint32_t p) {
+                        if constexpr (PREC == kPair) append_pair(list, cnt, a.cap, x, pb - p * pt, a.m_set);
+                        else append_raw(list, cnt, a.cap, b3, x, jb - p);
+                    };
                     // two appends by every lane, predicated (most slices give
                     // some lane two hits), their staging loads issued together;
                     // a loop for the rare third and later
@@ -468,14 +530,14 @@ __device__ __forceinline__ void tc_run(const CUtensorMap* tmap_q, const CUtensor
                         const uint32_t p1 = bfind31(h1);
                         const float x0 = stf[-static_cast<int>(p0)];
                         const float x1 = stf[-static_cast<int>(p1)];
-                        if (hits != 0u) append_raw(list, cnt, a.cap, b3, x0, jb - p0);
-                        if (h1 != 0u) append_raw(list, cnt, a.cap, b3, x1, jb - p1);
+                        if (hits != 0u) put_hit(x0, p0);
+                        if (h1 != 0u) put_hit(x1, p1);
                         hits = h1 & ~(1u << p1);
                     }
                     while (hits) {
                         const uint32_t p = bfind31(hits);
                         hits ^= 1u << p;
-                        append_raw(list, cnt, a.cap, b3, stf[-static_cast<int>(p)], jb - p);
+                        put_hit(stf[-static_cast<int>(p)], p);
                     }
                     // (each thread reads back only its own staging words: no
                     // warp barrier; the next tile's vote reconverges the warp)
@@ -581,6 +643,14 @@ tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CU
 
 // ------------------------------------------------ operand preparation kernels
 template <int PREC>
+__device__ __forceinline__ float lowp_round(float v) {
+    if (PREC == kBF16) return __bfloat162float(__float2bfloat16_rn(v));
+    uint32_t b;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(b) : "f"(v));
+    return __uint_as_float(b);
+}
+
+template <int PREC>
 __device__ __forceinline__ void put(void* row, int t, float v) {
     if (PREC == kBF16) {
         reinterpret_cast<__nv_bfloat16*>(row)[t] = __float2bfloat16_rn(v);
@@ -590,6 +660,189 @@ __device__ __forceinline__ void put(void* row, int t, float v) {
         reinterpret_cast<uint32_t*>(row)[t] = b;
     }
 }
+// ---- float32 rows as pairs of bf16 words
+//
+// The float32 search's own filter: three bf16 products in place of one fused
+// multiply-add per coordinate on the CUDA cores (33 TFLOP/s of 80, bound by
+// that pipe).  n = m = 38400, d = 96: 19 MMA steps of 16 coordinates a tile,
+// filter 0.79 ms, the whole search 8.57 -> 1.08 ms; n = 4999, m = 20011, d =
+// 50: 778 -> 116 us.  Two parts, not three: the part left out moves acc by less
+// than the slack any float32 bound over d terms has to carry, and the answer
+// is made of exact float32 distances either way (its error against float64 is
+// the same to the digit).
+//
+// x = h + l + e with h = bf16(x), l = bf16(x - h), |l| <= 2^-8 |x| and
+// |e| <= 2^-16 |x|.  The three products h.h + l.h + h.l on the tensor cores
+// leave out at most 3.01 * 2^-16 sum |q_t r_t| of q.r, and sum |q_t r_t| <=
+// (n_q + n_r) / 2 with n the squared norms: 1.505 * 2^-16 (n_q + n_r).
+//
+// Row layout (elements): h words [0, 16 hs), l words [16 hs, 32 hs), hs =
+// ceil(d / 16); five more words -- the reference's norm in three parts
+// against ones, ones against the query's threshold in two -- in the padding of
+// the h words when they fit (the l words there are zero, so they meet only
+// their own kind), else in one more K step.
+__host__ __device__ constexpr int kPairAug = 5;
+__host__ __device__ constexpr int pair_hsteps(int d) { return (d + 15) / 16; }
+__host__ __device__ constexpr bool pair_aug_inside(int d) { return d + kPairAug <= 16 * pair_hsteps(d); }
+__host__ __device__ constexpr int pair_aug(int d) {
+    return pair_aug_inside(d) ? d : 32 * pair_hsteps(d);
+}
+__host__ __device__ constexpr int pair_ksteps(int d) {
+    return 2 * pair_hsteps(d) + (pair_aug_inside(d) ? 0 : 1);
+}
+
+// Error bound of acc = q'.r' - n_r/2 + t as the tensor cores return it, as
+// eq n_q + er n_r + acc |t|.  Besides the words left out: each of the
+// 3 hs + 1 MMA steps adds 16 exact products to the accumulator, 17 addends each
+// cut at no less than 2^-23 of the largest partial sum, which is at most
+// 1.02 (n_q + n_r) / 2 + n_r / 2 + |t|; the norms are float32 sums of d squares
+// ((d + 8) 2^-24), cut to 24 bits; and taking q and r relative to a centre
+// rounds each coordinate once, 4 * 2^-24 (n_q + n_r) of the squared distance.
+struct PairSlack {
+    float eq, er, acc;
+};
+__host__ __device__ inline PairSlack pair_slack(int d) {
+    constexpr float u = 5.9604644775390625e-8f;   // 2^-24
+    PairSlack s;
+    s.acc = 34.f * u * static_cast<float>(3 * pair_hsteps(d) + 1);
+    const float common = 1.505f * 256.f * u + static_cast<float>(d + 16) * u;
+    s.eq = common + 0.51f * s.acc;
+    s.er = common + 1.02f * s.acc;
+    return s;
+}
+
+__device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+constexpr int kPairRows = 4;   // rows per warp
+constexpr int kPairMaxD = 192;
+
+// Operand rows of a search on pairs, references and queries in one launch:
+// warps below ref_warps take four consecutive rows of the reference copy, the
+// others four queries.  Coordinates are taken relative to the set's first
+// reference, so the slack follows the data's spread, not its offset from the
+// origin.  Row p of the copy, column c of tile g, holds reference
+// ((c mod 64) 4 + c / 64) T + g: every tile is an evenly spaced sample of the
+// whole set, and neighbours in storage order go to different column groups, so
+// a set stored cluster by cluster gives the pilot's sample and the hit lists
+// the same shares as a shuffled one.  Rows past the set get a norm word no
+// threshold passes.
+// The kernel reads and writes each row once, so memory bounds it; a lane holds
+// two neighbouring coordinates and stores them as one 32-bit word of h and one
+// of l, whole 128-byte lines per warp, and all loads of four rows are issued
+// before the first is used.  It also clears the search's two queue counters.
+__global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int64_t tiles,
+                                    const float* __restrict__ Q, int64_t n, int32_t d, int32_t kp,
+                                    uint32_t* __restrict__ R_lp, uint32_t* __restrict__ Q_lp,
+                                    float* __restrict__ qnorm, int64_t ref_warps,
+                                    int32_t* __restrict__ count0, int32_t* __restrict__ count1) {
+    constexpr int RW = kPairRows, NJ = kPairMaxD / 64;
+    const int lane = threadIdx.x % 32;
+    int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) / 32;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *count0 = 0;
+        *count1 = 0;
+    }
+    const bool ref = w < ref_warps;
+    if (!ref) w -= ref_warps;
+    const int64_t p0 = w * RW;
+    const int64_t rows = ref ? tiles * kTileN : n;
+    if (p0 >= rows) return;
+    const float* X = ref ? R : Q;
+    int64_t src[RW];
+#pragma unroll
+    for (int u = 0; u < RW; ++u) {
+        const int64_t p = p0 + u;
+        if (ref) {
+            const int c = static_cast<int>(p % kTileN);
+            src[u] = static_cast<int64_t>((c % kGroupCols) * kGroups + c / kGroupCols) * tiles + p / kTileN;
+            if (src[u] >= m) src[u] = -1;
+        } else {
+            src[u] = p < n ? p : -1;
+        }
+    }
+    float xv[RW][NJ][2];
+#pragma unroll
+    for (int u = 0; u < RW; ++u)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int t = 2 * lane + 64 * j + b;
+                xv[u][j][b] = (src[u] >= 0 && t < d) ? __ldg(X + src[u] * d + t) : 0.f;
+            }
+    float nr[RW];
+#pragma unroll
+    for (int u = 0; u < RW; ++u) nr[u] = 0.f;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int t = 2 * lane + 64 * j + b;
+            if (t < d) {
+                const float c = __ldg(R + t);
+#pragma unroll
+                for (int u = 0; u < RW; ++u) {
+                    if (src[u] >= 0) {
+                        xv[u][j][b] -= c;
+                        nr[u] = fmaf(xv[u][j][b], xv[u][j][b], nr[u]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < RW; ++u) nr[u] += __shfl_xor_sync(0xffffffffu, nr[u], o);
+    const int hs = pair_hsteps(d);
+    const bool inside = pair_aug_inside(d);
+    const float half_er = 0.5f - pair_slack(d).er;   // -(1/2 - er) n_r: er n_r of slack on acc
+#pragma unroll
+    for (int u = 0; u < RW; ++u) {
+        const int64_t p = p0 + u;
+        if (p >= rows) break;
+        float aug[kPairAug];
+        if (ref) {
+            // -(1 - 2 er) n_r / 2 in three parts
+            const float v = src[u] >= 0 ? -half_er * nr[u] : -3e38f;
+            aug[0] = lowp_round<kBF16>(v);
+            aug[1] = lowp_round<kBF16>(v - aug[0]);
+            aug[2] = (v - aug[0]) - aug[1];
+            aug[3] = aug[4] = 1.f;
+            if (src[u] < 0) aug[1] = aug[2] = 0.f;
+        } else {
+            aug[0] = aug[1] = aug[2] = 1.f;
+            aug[3] = aug[4] = 0.f;
+            if (lane == 0) qnorm[p] = nr[u];
+        }
+        auto aug_at = [&](int i) {   // the i-th extra word, 0 outside
+            float v = 0.f;
+#pragma unroll
+            for (int x = 0; x < kPairAug; ++x) v = i == x ? aug[x] : v;
+            return v;
+        };
+        uint32_t* row = (ref ? R_lp : Q_lp) + p * (kp / 2);
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const int t = 2 * lane + 64 * j;
+            if (t >= 16 * hs) break;
+            const float x0 = xv[u][j][0], x1 = xv[u][j][1];
+            float h0 = lowp_round<kBF16>(x0), h1 = lowp_round<kBF16>(x1);
+            row[8 * hs + t / 2] = bf16x2_bits(t < d ? x0 - h0 : 0.f, t + 1 < d ? x1 - h1 : 0.f);
+            if (inside) {
+                if (t >= d) h0 = aug_at(t - d);
+                if (t + 1 >= d) h1 = aug_at(t + 1 - d);
+            }
+            row[t / 2] = bf16x2_bits(h0, h1);
+        }
+        for (int e = 2 * lane; e < kp - 32 * hs; e += 64)
+            row[16 * hs + e / 2] =
+                inside ? 0u : bf16x2_bits(aug_at(e), aug_at(e + 1));
+    }
+}
+
 template <int PREC>
 __device__ __forceinline__ float get(const void* row, int t) {
     if (PREC == kBF16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(row)[t]);
@@ -615,14 +868,6 @@ __device__ __forceinline__ void put4(void* row, int t, float4 v) {
         reinterpret_cast<uint4*>(row)[t / 4] = w;
     }
 }
-template <int PREC>
-__device__ __forceinline__ float lowp_round(float v) {
-    if (PREC == kBF16) return __bfloat162float(__float2bfloat16_rn(v));
-    uint32_t b;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(b) : "f"(v));
-    return __uint_as_float(b);
-}
-
 // Smallest power of two >= x (x > 0, finite).
 __device__ __forceinline__ float pow2_ceil(float x) {
     return __uint_as_float((__float_as_uint(x) + 0x007fffffu) & 0x7f800000u);
@@ -764,6 +1009,13 @@ __global__ void prepare_kernel(const float* __restrict__ X, int64_t rows, int32_
 // >= prefix|bit at least cprime?) down to bit 8.  Stopping there leaves a
 // value at most 2^8 order steps (2^-15 relative) below the exact one: a
 // slightly lower threshold, so never fewer passing references.
+//
+// Operand pairs (PREC = kPair): qscale[q] holds the query's squared norm n_q;
+// in its place goes the bound that certifies the query's answer.  With the
+// norm words slack of the reference folded in (pair_slack), every reference
+// has ||q - r||^2 >= bound - 2 acc, so those that fail the filter are at least
+// `bound` away.  A query whose norm is not finite or above 1e36 (where float32
+// squares overflow) gets -inf: it is never certified.
 template <int PREC, int VPL>
 __device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gmax, int64_t q,
                                                 int32_t G, int32_t cprime, int32_t d, int32_t kp,
@@ -772,14 +1024,18 @@ __device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gma
                                                 float* __restrict__ qscale, int lane) {
     const uint32_t* src = gmax + q * G;
     // squared norm of the (low-precision) query row, for the hit-code scale
-    const size_t elt = (PREC == kBF16) ? 2 : 4;
+    const size_t elt = (PREC == kTF32) ? 4 : 2;
     void* row = static_cast<unsigned char*>(Q_lp) + static_cast<size_t>(q) * kp * elt;
     float nq2 = 0.f;
-    for (int t = lane; t < d; t += 32) {
-        const float x = get<PREC>(row, t);
-        nq2 = fmaf(x, x, nq2);
+    if constexpr (PREC == kPair) {
+        nq2 = qscale[q];
+    } else {
+        for (int t = lane; t < d; t += 32) {
+            const float x = get<PREC>(row, t);
+            nq2 = fmaf(x, x, nq2);
+        }
+        for (int o = 16; o > 0; o >>= 1) nq2 += __shfl_xor_sync(0xffffffffu, nq2, o);
     }
-    for (int o = 16; o > 0; o >>= 1) nq2 += __shfl_xor_sync(0xffffffffu, nq2, o);
     uint32_t v[VPL];
     uint32_t least = 0xffffffffu, most = 0u;
     int nvalid = 0;
@@ -810,6 +1066,25 @@ __device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gma
     }
     const uint32_t best = nvalid >= cprime ? prefix : least;   // fewer than cprime groups: the weakest
     const float t_acc = unord_f32(best);
+    if constexpr (PREC == kPair) {
+        const float tc = -t_acc + 1e-4f * fabsf(t_acc) + 1e-5f * nq2;
+        const float hi = lowp_round<kBF16>(tc);
+        const float lo = lowp_round<kBF16>(tc - hi);
+        if (lane == 0) {
+            const int at = pair_aug(d) + 3;
+            put<kBF16>(row, at, hi);
+            put<kBF16>(row, at + 1, lo);
+            const PairSlack ps = pair_slack(d);
+            const float t = hi + lo;
+            // float32 rounding of the four operations here: 8 and 16 units of
+            // 2^-24; squares that underflow: 1e-33
+            constexpr float u = 5.9604644775390625e-8f;
+            const float b = nq2 * (1.f - 2.f * ps.eq - 8.f * u) + 2.f * t -
+                            (2.f * ps.acc + 16.f * u) * fabsf(t) - 1e-33f;
+            qscale[q] = nq2 <= 1e36f ? b : __int_as_float(0xff800000);
+        }
+        return;
+    }
     const float tcol = -t_acc + 1e-3f * (1.f + fabsf(t_acc));
     const float hi = lowp_round<PREC>(tcol);
     const float lo = lowp_round<PREC>(tcol - hi);
