@@ -428,10 +428,13 @@ __device__ void gather_cand(const FinalizeArgs& a, int64_t q, WarpScratch& w, in
 // The score of a hit-list key: its high word, a code in [0, 0xffff] that
 // falls linearly with the low-precision score, as a float (exact: the code
 // sits in the mantissa of 2^23 + code).
-// PAIR (operand pairs): -acc, from a high word of 0x7f800000 minus acc's bits.
-template <bool PAIR>
+// Certified lists: operand pairs -acc, from a high word of 0x7f800000 minus
+// acc's bits; differences the distance itself.
+enum Cert : int { kNoCert = 0, kCertPair = 1, kCertDiff = 2 };
+template <int CERT>
 __device__ __forceinline__ float hit_val(uint32_t hi) {
-    if (PAIR) return -__uint_as_float(0x7f800000u - hi);
+    if (CERT == kCertPair) return -__uint_as_float(0x7f800000u - hi);
+    if (CERT == kCertDiff) return __uint_as_float(hi);
     return __uint_as_float(0x4B000000u | hi) - 8388608.f;
 }
 
@@ -501,11 +504,12 @@ __device__ __forceinline__ void hit_totals(const FinalizeArgs& a, int64_t q, int
 // pass reads shared memory; the kept indices are compacted in place, each
 // written at or before the position it was read from (MODE 2).  Longer ones
 // are re-read from global memory at every pass (MODE 0).
-// PAIR: *acc_cut becomes the largest acc among the listed references that
-// were not kept (0 when all were: those not listed have acc < 0).
-template <int METRIC, int NV, int MODE, bool PAIR>
+// CERT: *cut_out becomes the value (hit_val) of the nearest listed reference
+// that was not kept; 0 (pairs: those not listed have acc < 0) or +inf
+// (differences) when all were.
+template <int METRIC, int NV, int MODE, int CERT>
 __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScratch& w, int lane,
-                                int total, float* acc_cut) {
+                                int total, float* cut_out) {
     constexpr bool STAGED = MODE != 0;
     const HitLists& hl = a.hits;
     const int S = hl.S, cap = hl.cap, c = hl.c;
@@ -565,11 +569,11 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
         if constexpr (MODE == 1) {
 #pragma unroll
             for (int i = 0; i < kRegHits; ++i)
-                if (i * 32 + lane < total) f(hit_val<PAIR>(hv[i]));
+                if (i * 32 + lane < total) f(hit_val<CERT>(hv[i]));
         } else if constexpr (MODE == 2) {
-            for (int e = lane; e < total; e += 32) f(hit_val<PAIR>(static_cast<uint32_t>(w.keys[e] >> 32)));
+            for (int e = lane; e < total; e += 32) f(hit_val<CERT>(static_cast<uint32_t>(w.keys[e] >> 32)));
         } else {
-            visit_global([&](uint64_t key) { f(hit_val<PAIR>(static_cast<uint32_t>(key >> 32))); });
+            visit_global([&](uint64_t key) { f(hit_val<CERT>(static_cast<uint32_t>(key >> 32))); });
         }
     };
     for_each([&](float v) {
@@ -612,16 +616,16 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
         return bb < cut1 || (bb == cut1 && (b2.inv == 0.f || b2.bin(v) <= cut2));
     };
     int kept = 0;
-    float cut = 0.f;   // -acc of the best reference this lane cut, 0 at most
+    float cut = CERT == kCertDiff ? __int_as_float(0x7f800000) : 0.f;   // nearest this lane cut
     if constexpr (MODE == 2) {
         // in place: every lane reads its entry before any lane writes, and a
         // kept entry goes to a position at or before the one it came from
         for (int e0 = 0; e0 < total; e0 += 32) {
             const int e = e0 + lane;
             const uint64_t key = e < total ? w.keys[e] : 0ull;
-            const float v = hit_val<PAIR>(static_cast<uint32_t>(key >> 32));
+            const float v = hit_val<CERT>(static_cast<uint32_t>(key >> 32));
             const bool take = e < total && keep(v);
-            if (PAIR && e < total && !take) cut = fminf(cut, v);
+            if (CERT && e < total && !take) cut = fminf(cut, v);
             const unsigned bal = __ballot_sync(0xffffffffu, take);
             __syncwarp();
             const int pos = kept + __popc(bal & ((1u << lane) - 1u));
@@ -633,9 +637,9 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
 #pragma unroll
         for (int i = 0; i < kRegHits; ++i) {
             const int e = i * 32 + lane;
-            const float v = hit_val<PAIR>(hv[i]);
+            const float v = hit_val<CERT>(hv[i]);
             const bool take = e < total && keep(v);
-            if (PAIR && e < total && !take) cut = fminf(cut, v);
+            if (CERT && e < total && !take) cut = fminf(cut, v);
             const unsigned bal = __ballot_sync(0xffffffffu, take);
             const int pos = kept + __popc(bal & ((1u << lane) - 1u));
             if (take && pos < P) w.keys[pos] = static_cast<uint32_t>(w.stage[e]);
@@ -645,11 +649,11 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
         if (lane == 0) w.hist[kBins] = 0;
         __syncwarp();
         visit_global([&](uint64_t key) {
-            const float v = hit_val<PAIR>(static_cast<uint32_t>(key >> 32));
+            const float v = hit_val<CERT>(static_cast<uint32_t>(key >> 32));
             if (keep(v)) {
                 const int pos = atomicAdd(&w.hist[kBins], 1);
                 if (pos < P) w.keys[pos] = key_idx(key);
-            } else if (PAIR) {
+            } else if (CERT) {
                 cut = fminf(cut, v);
             }
         });
@@ -658,9 +662,9 @@ __device__ int gather_hits_impl(const FinalizeArgs& a, int64_t q, int P, WarpScr
     }
     __syncwarp();
     if (kept > P) return -3;
-    if (PAIR) {
+    if (CERT) {
         for (int o = 16; o > 0; o >>= 1) cut = fminf(cut, __shfl_xor_sync(0xffffffffu, cut, o));
-        *acc_cut = -cut;
+        *cut_out = cut;
     }
     exact_keys<METRIC, NV>(w.keys, kept, a.R, a.d, w.qrow, lane);
     return kept;
@@ -704,9 +708,9 @@ __device__ __forceinline__ void queue_fallback(const FinalizeArgs& a, int64_t q,
 // shared memory (warp_scratch_bytes for these P, S, d and staging entries).
 // Every step is warp-synchronous; nothing waits on the rest of the CTA.
 // crow: the query's row of the candidate set (q unless the pass runs over a
-// queue).  PAIR: hit lists of an operand-pair filter, whose answers are
-// certified by the list's bound.
-template <int METRIC, int NV, bool PAIR = false>
+// queue).  CERT: hit lists of a float32 filter, whose answers are certified by
+// the lists' bound.
+template <int METRIC, int NV, int CERT = kNoCert>
 __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, int64_t q,
                                unsigned char* scratch, int lane, int64_t crow) {
     const int S = a.use_hits ? 1 : a.cand.S;
@@ -735,17 +739,17 @@ __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, 
 
     // 1. candidates with exact float32 keys
     int pool;
-    float acc_cut = 0.f;
+    float cut = 0.f;
     if (!a.use_hits) {
         pool = a.cand.S * a.cand.c;
         gather_cand<METRIC, NV>(a, crow, w, lane);
     } else {
         if (over) pool = -2;
         else if (total < a.hits.c && total < a.m) pool = -1;
-        else if (total <= kStage) pool = gather_hits_impl<METRIC, NV, 1, PAIR>(a, q, P, w, lane, total, &acc_cut);
+        else if (total <= kStage) pool = gather_hits_impl<METRIC, NV, 1, CERT>(a, q, P, w, lane, total, &cut);
         else if (total <= stage_all)
-            pool = gather_hits_impl<METRIC, NV, 2, PAIR>(a, q, P, w, lane, total, &acc_cut);
-        else pool = gather_hits_impl<METRIC, NV, 0, PAIR>(a, q, P, w, lane, total, &acc_cut);
+            pool = gather_hits_impl<METRIC, NV, 2, CERT>(a, q, P, w, lane, total, &cut);
+        else pool = gather_hits_impl<METRIC, NV, 0, CERT>(a, q, P, w, lane, total, &cut);
         if (pool < 0) {
             if (lane == 0) queue_fallback(a, q, -pool - 1);
             return;
@@ -926,10 +930,12 @@ __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, 
         return (w.runs[kk - 1] >= 0) ? static_cast<double>(refined(w.d64[sk])) * (1.0 + 1e-6)
                                      : static_cast<double>(key_dist(w.sorted[sk])) * (1.0 + a.rel);
     };
-    // 4. completeness.  Operand pairs: the references that were not kept have
-    //    acc <= acc_cut, so they are at least bound - 2 acc_cut away
-    if (PAIR) {
-        const double lower = static_cast<double>(a.hits.bound[q]) - 2.0 * static_cast<double>(acc_cut);
+    // 4. completeness of a certified list.  Operand pairs: the references that
+    //    were not kept have -acc >= cut, so they are at least bound + 2 cut away;
+    //    differences: they are at least as far as the nearer of bound and cut
+    if (CERT) {
+        const double b = static_cast<double>(a.hits.bound[q]), v = static_cast<double>(cut);
+        const double lower = CERT == kCertPair ? b + 2.0 * v : fmin(b, v) * (1.0 - a.rel);
         if (kk < k || !(lower > kth_upper())) {
             if (lane == 0) queue_fallback(a, q, 3);
             return;
@@ -979,7 +985,7 @@ __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, 
     }
 }
 
-template <int METRIC, int NV, bool PAIR>
+template <int METRIC, int NV, int CERT>
 __global__ void __launch_bounds__(kFinThreads, 4)
 finalize_kernel(FinalizeArgs a, int P, int warps_per_block, int stage_entries) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -989,7 +995,7 @@ finalize_kernel(FinalizeArgs a, int P, int warps_per_block, int stage_entries) {
     if (a.fb_done && blockIdx.x == 0 && static_cast<int>(threadIdx.x) < a.fb_slots)
         a.fb_done[threadIdx.x] = 0;   // the fallback's chunk counters, for this search
     if (q >= a.n) return;   // warp-uniform: no block-level sync below
-    if (!PAIR && a.from.list) {
+    if (!CERT && a.from.list) {
         const int count = *a.from.count;
         if (row >= count) return;
         q = a.from.list[row];
@@ -1001,7 +1007,7 @@ finalize_kernel(FinalizeArgs a, int P, int warps_per_block, int stage_entries) {
     const int S = a.use_hits ? 1 : a.cand.S;
     const size_t per_warp =
         warp_scratch_bytes(P, prefix_cap(P, a.k), S, a.d, a.use_hits ? stage_entries : 0);
-    finalize_query<METRIC, NV, PAIR>(a, P, stage_entries, q, smem_raw + per_warp * warp, lane, row);
+    finalize_query<METRIC, NV, CERT>(a, P, stage_entries, q, smem_raw + per_warp * warp, lane, row);
 }
 
 // ---------------------------------------------------------------------------

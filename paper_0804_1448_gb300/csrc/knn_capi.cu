@@ -30,7 +30,7 @@ constexpr int64_t kPartMinQueries = 4096;
 // The most workspace a search may plan for its operand-pair filter.  Ten
 // million queries against 5000 references would hold 41 GB of hit lists for
 // what the select does in 3; a set of four million, d = 128, needs 3 GB.
-constexpr size_t kPairMaxBytes = 16ull << 30;
+constexpr size_t kFilterMaxBytes = 16ull << 30;
 
 // Device counters owned by a handle.
 struct Counters {
@@ -313,6 +313,11 @@ struct SearchPlan {
     // the tensor-core slices below are its own); S, chunk and c stay those of
     // the CUDA-core select, which takes the queries the filter cannot certify
     bool pair = false;
+    // float32, Manhattan and Chebyshev: the filter on differences runs first
+    // (dplan), the queries it cannot certify likewise
+    bool diff = false;
+    DiffPlan dplan{};
+    bool filtered() const { return pair || diff; }
     int c_need = 0;          // small: the nearest keys a query must keep (c slots, c >= c_need)
     int prec = 0;
     int kp = 0;
@@ -349,7 +354,7 @@ bool plan_pair(int64_t n, int64_t m, int32_t d, int32_t c, int sm_share, SearchP
 // lone search; fewer when several run side by side in a batch).
 knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision, int64_t n, int32_t k,
                           knn_metric metric, int io_on_device, int sm_share, SearchPlan* sp,
-                          int64_t fb_cap_bytes = 64LL << 20, bool allow_pair = true) {
+                          int64_t fb_cap_bytes = 64LL << 20, bool allow_filter = true) {
     SearchPlan p;
     p.tensor = (metric == KNN_L2) && precision != KNN_FP32;
     p.prec = p.tensor ? (precision == KNN_BF16 ? kBF16 : kTF32) : 0;
@@ -386,7 +391,7 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
         if (p.plan.stages == 0 ||
             (small_select_fits(m, d) && (!p.plan.pilot || small_share < kSmallSelectShare)))
             return plan_search_md(h, m, d, KNN_FP32, n, k, metric, io_on_device, sm_share, sp,
-                                  fb_cap_bytes, allow_pair);
+                                  fb_cap_bytes, allow_filter);
         p.S = p.plan.S;
         p.chunk = p.plan.chunk;
     } else if (small_select_fits(m, d)) {
@@ -401,7 +406,11 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
         if (static_cast<int64_t>(S) * p.c > finalize_max_pool()) return KNN_ERR_UNSUPPORTED;
         p.S = S;
         p.chunk = chunk;
-        p.pair = allow_pair && metric == KNN_L2 && plan_pair(n, m, d, p.c, sm_share, &p);
+        p.pair = allow_filter && metric == KNN_L2 && plan_pair(n, m, d, p.c, sm_share, &p);
+        if (allow_filter && metric != KNN_L2 && 2 * p.c + 32 <= finalize_max_pool()) {
+            p.dplan = diff_plan(n, m, d, p.c, sm_share);
+            p.diff = p.dplan.pilot;
+        }
     }
 
     // fallback grid: scratch of grid * m doubles, at most fb_cap_bytes
@@ -411,10 +420,8 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
 
     // workspace layout
     Carve cv;
-    if (p.pair) {
-        p.off_rl = cv.take(static_cast<size_t>(pair_tiles(m)) * kPairTile * p.kp * 2);
-        p.off_queue = cv.take((static_cast<size_t>(n) + 1) * sizeof(int32_t));
-    }
+    if (p.pair) p.off_rl = cv.take(static_cast<size_t>(pair_tiles(m)) * kPairTile * p.kp * 2);
+    if (p.filtered()) p.off_queue = cv.take((static_cast<size_t>(n) + 1) * sizeof(int32_t));
     if (p.tensor || p.pair) {
         const size_t elt = p.prec == kTF32 ? 4 : 2;
         p.off_ql = cv.take(static_cast<size_t>(n) * p.kp * elt);
@@ -427,6 +434,14 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
         p.off_lists = cv.take(list_bytes);
         p.off_cand = p.off_lists;
         p.off_counts = cv.take(static_cast<size_t>(n) * p.plan.S * p.plan.groups * sizeof(int32_t));
+        p.off_qs = cv.take(static_cast<size_t>(n) * sizeof(float));
+    } else if (p.diff) {
+        const DiffPlan& dp = p.dplan;
+        p.off_gmax = cv.take(static_cast<size_t>(n) * dp.G * 4);
+        p.off_lists = cv.take(std::max(static_cast<size_t>(n) * dp.S * dp.cap * sizeof(uint64_t),
+                                       static_cast<size_t>(n) * p.S * p.c * sizeof(uint64_t)));
+        p.off_cand = p.off_lists;
+        p.off_counts = cv.take(static_cast<size_t>(n) * dp.S * sizeof(int32_t));
         p.off_qs = cv.take(static_cast<size_t>(n) * sizeof(float));
     } else {
         p.off_cand = cv.take(static_cast<size_t>(n) * p.S * p.c * sizeof(uint64_t));
@@ -441,11 +456,11 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
     }
     p.bytes = cv.off;
     // the filter's copies and lists are scratch the select alone does not need:
-    // it runs alone where they would pass the handle's limit, or kPairMaxBytes
+    // it runs alone where they would pass the handle's limit, or kFilterMaxBytes
     const size_t most = h->opt.workspace_limit > 0
-                            ? std::min(kPairMaxBytes, static_cast<size_t>(h->opt.workspace_limit))
-                            : kPairMaxBytes;
-    if (p.pair && p.bytes > most)
+                            ? std::min(kFilterMaxBytes, static_cast<size_t>(h->opt.workspace_limit))
+                            : kFilterMaxBytes;
+    if (p.filtered() && p.bytes > most)
         return plan_search_md(h, m, d, precision, n, k, metric, io_on_device, sm_share, sp,
                               fb_cap_bytes, false);
     *sp = p;
@@ -453,20 +468,20 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
 }
 
 knn_status plan_search(const knn_ctx* h, int64_t n, int32_t k, knn_metric metric, int io_on_device,
-                       SearchPlan* sp, bool allow_pair = true) {
+                       SearchPlan* sp, bool allow_filter = true) {
     return plan_search_md(h, h->ref->m, h->ref->d, h->opt.precision, n, k, metric, io_on_device,
-                          h->num_sms, sp, 64LL << 20, allow_pair);
+                          h->num_sms, sp, 64LL << 20, allow_filter);
 }
 
 // Plan a search on st and hold its workspace, `extra` bytes after the plan's
-// own included.  A float32 search whose operand-pair scratch cannot be had --
+// own included.  A float32 search whose filter's scratch cannot be had --
 // no memory, or a capturing stream and a workspace that would have to grow --
 // runs the select alone, which needs less.
 knn_status plan_and_hold(knn_ctx* h, int64_t n, int32_t k, knn_metric metric, int io_on_device,
                          cudaStream_t st, size_t extra, SearchPlan* sp) {
     knn_status s = plan_search(h, n, k, metric, io_on_device, sp);
     if (s != KNN_OK) return s;
-    if (sp->pair && sp->bytes + extra > h->ws_bytes) {
+    if (sp->filtered() && sp->bytes + extra > h->ws_bytes) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         KNN_CUDA(h, cudaStreamIsCapturing(st, &cap));
         s = cap == cudaStreamCaptureStatusNone ? ensure_workspace(h, sp->bytes + extra) : KNN_ERR_OOM;
@@ -506,7 +521,7 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
     };
     FinalizeArgs fa{};
     QueryQueue queue{};
-    if (sp.pair) {
+    if (sp.filtered()) {
         queue.count = reinterpret_cast<int32_t*>(ws + sp.off_queue);
         queue.list = queue.count + 1;
     } else {
@@ -554,6 +569,28 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
         fa.cand.exact = 0;
         fa.cand.S = 1;
         fa.cand.c = c;
+    } else if (sp.diff) {
+        const DiffPlan& dp = sp.dplan;
+        uint32_t* gmax = reinterpret_cast<uint32_t*>(ws + sp.off_gmax);
+        float* thr = reinterpret_cast<float*>(ws + sp.off_qs);
+        uint64_t* lists = reinterpret_cast<uint64_t*>(ws + sp.off_lists);
+        int32_t* counts = reinterpret_cast<int32_t*>(ws + sp.off_counts);
+        KNN_CUDA(h, launch_diff_pilot(dp, Qd, n, rv.R, m, d, metric, gmax, st, l));
+        mark("diff_pilot");
+        KNN_CUDA(h, launch_diff_threshold(dp, gmax, n, thr, queue.count, fallback_count, st, l));
+        mark("diff_threshold");
+        KNN_CUDA(h, launch_diff_filter(dp, Qd, n, rv.R, m, d, metric, thr, lists, counts, st, l));
+        mark("diff_filter");
+        fa.use_hits = 1;
+        fa.hits.keys = lists;
+        fa.hits.counts = counts;
+        fa.hits.S = dp.S;
+        fa.hits.cap = dp.cap;
+        fa.hits.c = c;
+        fa.hits.bound = thr;
+        fa.cand.exact = 0;
+        fa.cand.S = 1;
+        fa.cand.c = c;
     } else {
         CandidateSet cs;
         cs.keys = reinterpret_cast<uint64_t*>(ws + sp.off_cand);
@@ -588,7 +625,7 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
     fa.fallback_reason = ctr->fallback_reason;
     fa.fb_done = reinterpret_cast<int32_t*>(ws + sp.off_fbdone);
     fa.fb_slots = static_cast<int32_t>(sp.fb_grid);
-    if (sp.pair) {
+    if (sp.filtered()) {
         // the filter's answers; the queries it cannot certify go through the
         // CUDA-core select (a few: straight to the exact fallback)
         FinalizeArgs fp = fa;

@@ -13,6 +13,11 @@
 // so the serial part of the selection shrinks to the rare insertions.  Only
 // the c survivors per (query, split) are written out.
 //
+// Most float32 searches run a filter instead (operand pairs on the tensor
+// cores, knn_tc.cu; Manhattan and Chebyshev, knn_diff.cu).  This form takes
+// what they cannot: rows too long for them, workspace limits, batches, and the
+// queries a filter leaves over (a queue).
+//
 // Manhattan and Chebyshev distances are formed from coordinate differences in
 // float32, coordinate 0 first (sum_t |q_t - r_t|, max_t |q_t - r_t|).  The
 // Euclidean one is expanded, ||q - r||^2 = ||q||^2 + ||r||^2 - 2 q.r: one
@@ -441,6 +446,18 @@ cudaError_t launch_rows(const float* Q, int64_t n, const float* R, int64_t m, in
     return cudaGetLastError();
 }
 
+template <int METRIC>
+cudaError_t launch_metric(int rows, const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
+                          const CandidateSet& cand, cudaStream_t st, const QueryQueue& from) {
+    if (from.list)
+        return rows == 128 ? launch_rows<METRIC, 128, true>(Q, n, R, m, d, cand, st, from)
+               : rows == 64 ? launch_rows<METRIC, 64, true>(Q, n, R, m, d, cand, st, from)
+                            : launch_rows<METRIC, 16, true>(Q, n, R, m, d, cand, st, from);
+    return rows == 128 ? launch_rows<METRIC, 128>(Q, n, R, m, d, cand, st)
+           : rows == 64 ? launch_rows<METRIC, 64>(Q, n, R, m, d, cand, st)
+                        : launch_rows<METRIC, 16>(Q, n, R, m, d, cand, st);
+}
+
 constexpr size_t kSmemCap = 220 * 1024;
 constexpr size_t kSmemPerSm = 233472;   // shared memory of one SM
 constexpr size_t kSmemPerCta = 1024;    // reserved by the hardware per resident CTA
@@ -523,23 +540,9 @@ cudaError_t launch_cc_select(const float* Q, int64_t n, const float* R, int64_t 
     const int rows = cc_rows(n, cand.c, &per_sm);
     if (rows == 16 && cc_smem_bytes<16>(cand.c) > kSmemCap) return cudaErrorInvalidValue;
     if (launches) ++*launches;
-    if (from.list) {
-        if (metric != kL2) return cudaErrorInvalidValue;
-        return rows == 128 ? launch_rows<kL2, 128, true>(Q, n, R, m, d, cand, st, from)
-               : rows == 64 ? launch_rows<kL2, 64, true>(Q, n, R, m, d, cand, st, from)
-                            : launch_rows<kL2, 16, true>(Q, n, R, m, d, cand, st, from);
-    }
-    if (metric == kL2)
-        return rows == 128 ? launch_rows<kL2, 128>(Q, n, R, m, d, cand, st)
-               : rows == 64 ? launch_rows<kL2, 64>(Q, n, R, m, d, cand, st)
-                            : launch_rows<kL2, 16>(Q, n, R, m, d, cand, st);
-    if (metric == kL1)
-        return rows == 128 ? launch_rows<kL1, 128>(Q, n, R, m, d, cand, st)
-               : rows == 64 ? launch_rows<kL1, 64>(Q, n, R, m, d, cand, st)
-                            : launch_rows<kL1, 16>(Q, n, R, m, d, cand, st);
-    return rows == 128 ? launch_rows<kLinf, 128>(Q, n, R, m, d, cand, st)
-           : rows == 64 ? launch_rows<kLinf, 64>(Q, n, R, m, d, cand, st)
-                        : launch_rows<kLinf, 16>(Q, n, R, m, d, cand, st);
+    if (metric == kL2) return launch_metric<kL2>(rows, Q, n, R, m, d, cand, st, from);
+    if (metric == kL1) return launch_metric<kL1>(rows, Q, n, R, m, d, cand, st, from);
+    return launch_metric<kLinf>(rows, Q, n, R, m, d, cand, st, from);
 }
 
 }  // namespace knn

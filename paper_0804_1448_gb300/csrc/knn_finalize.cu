@@ -33,24 +33,24 @@ cudaError_t launch_drop_self(const float* din, const int32_t* iin, int64_t n, in
 
 int finalize_max_pool() { return kMaxPool; }
 
-template <int METRIC, int NV, bool PAIR>
+template <int METRIC, int NV, int CERT>
 cudaError_t launch_finalize_nv(const FinalizeArgs& a, int P, int wpb, int se, size_t smem,
                                unsigned grid, cudaStream_t st) {
-    cudaError_t err = allow_smem<finalize_kernel<METRIC, NV, PAIR>>(smem);
+    cudaError_t err = allow_smem<finalize_kernel<METRIC, NV, CERT>>(smem);
     if (err != cudaSuccess) return err;
-    finalize_kernel<METRIC, NV, PAIR><<<grid, wpb * 32, smem, st>>>(a, P, wpb, se);
+    finalize_kernel<METRIC, NV, CERT><<<grid, wpb * 32, smem, st>>>(a, P, wpb, se);
     return cudaGetLastError();
 }
 
-template <int METRIC, bool PAIR = false>
+template <int METRIC, int CERT = kNoCert>
 cudaError_t launch_finalize_m(const FinalizeArgs& a, int nv, int P, int wpb, int se, size_t smem,
                               unsigned grid, cudaStream_t st) {
     switch (nv) {
-        case 1: return launch_finalize_nv<METRIC, 1, PAIR>(a, P, wpb, se, smem, grid, st);
-        case 2: return launch_finalize_nv<METRIC, 2, PAIR>(a, P, wpb, se, smem, grid, st);
-        case 3: return launch_finalize_nv<METRIC, 3, PAIR>(a, P, wpb, se, smem, grid, st);
-        case 4: return launch_finalize_nv<METRIC, 4, PAIR>(a, P, wpb, se, smem, grid, st);
-        default: return launch_finalize_nv<METRIC, 0, PAIR>(a, P, wpb, se, smem, grid, st);
+        case 1: return launch_finalize_nv<METRIC, 1, CERT>(a, P, wpb, se, smem, grid, st);
+        case 2: return launch_finalize_nv<METRIC, 2, CERT>(a, P, wpb, se, smem, grid, st);
+        case 3: return launch_finalize_nv<METRIC, 3, CERT>(a, P, wpb, se, smem, grid, st);
+        case 4: return launch_finalize_nv<METRIC, 4, CERT>(a, P, wpb, se, smem, grid, st);
+        default: return launch_finalize_nv<METRIC, 0, CERT>(a, P, wpb, se, smem, grid, st);
     }
 }
 
@@ -84,8 +84,11 @@ cudaError_t launch_finalize(const FinalizeArgs& a_in, cudaStream_t st, int* laun
         ((reinterpret_cast<uintptr_t>(a.R) | reinterpret_cast<uintptr_t>(a.Q)) & 15) == 0;
     const int nv = (aligned && (a.d & 3) == 0 && a.d <= 128) ? (a.d + 31) / 32 : 0;
     if (launches) ++*launches;
-    if (a.use_hits && a.hits.bound)
-        return launch_finalize_m<kL2, true>(a, nv, P, wpb, se, smem, grid, st);
+    if (a.use_hits && a.hits.bound) {
+        if (a.metric == kL2) return launch_finalize_m<kL2, kCertPair>(a, nv, P, wpb, se, smem, grid, st);
+        if (a.metric == kL1) return launch_finalize_m<kL1, kCertDiff>(a, nv, P, wpb, se, smem, grid, st);
+        return launch_finalize_m<kLinf, kCertDiff>(a, nv, P, wpb, se, smem, grid, st);
+    }
     if (a.metric == kL2) return launch_finalize_m<kL2>(a, nv, P, wpb, se, smem, grid, st);
     if (a.metric == kL1) return launch_finalize_m<kL1>(a, nv, P, wpb, se, smem, grid, st);
     return launch_finalize_m<kLinf>(a, nv, P, wpb, se, smem, grid, st);

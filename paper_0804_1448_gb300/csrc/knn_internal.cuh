@@ -12,6 +12,8 @@
 //                  A float32 Euclidean search takes the tensor-core form on
 //                  pairs of bf16 words, whose answers the finalize certifies;
 //                  the queries it cannot certify take the CUDA-core form.
+//                  Manhattan and Chebyshev searches likewise filter on CUDA
+//                  cores first (knn_diff.cu).
 //   2. finalize -- per query: exact float32 distances of the candidates, a sort
 //                  by (distance, index), a float64 re-check of candidates whose
 //                  float32 distances are within rounding of each other, and the
@@ -110,9 +112,12 @@ struct HitLists {
     int32_t S;
     int32_t cap;
     int32_t c;              // keep (at least) the best c before the exact re-rank
-    const float* bound;     // operand pairs: [n], every reference is at least bound - 2 acc
-                            // away (squared), and the keys' high word is 0x7f800000 minus
-                            // the bits of acc, 0 for a reference not listed; else null
+    // float32 searches, whose answers are certified (else null): [n].
+    // Operand pairs: every reference is at least bound - 2 acc away (squared),
+    // acc < 0 for those not listed; the keys' high word is 0x7f800000 minus the
+    // bits of acc.  Differences: those not listed are farther than bound; the
+    // high word is the bits of the distance.
+    const float* bound;
 };
 
 // The queries one pass left to the next: list[0 .. *count).  A pass over a
@@ -156,11 +161,36 @@ struct FinalizeArgs {
 // ---- launchers (return cudaSuccess or the launch error) -------------------
 
 // CUDA-core fused distance + top-c.  Writes cand (exact = 1).
-// from.list: only the queue's queries (Euclidean), candidate row i being that
+// from.list: only the queue's queries, candidate row i being that
 // of its i-th.
 cudaError_t launch_cc_select(const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
                              int32_t metric, const CandidateSet& cand, cudaStream_t st,
                              int* launches, const QueryQueue& from = QueryQueue{});
+
+// Manhattan and Chebyshev searches with a pilot threshold and hit lists
+// (knn_diff.cu), one list per query and split.
+struct DiffPlan {
+    int32_t rows;        // queries per CTA: 128, 64 or 16 (0: rows too long)
+    int32_t tiles;       // 128-reference tiles of the set
+    int32_t tps;         // tiles per split
+    int32_t S;           // reference splits
+    int32_t stride;      // pilot samples every stride-th tile of the set
+    int32_t spt;         // sampled tiles per pilot CTA
+    int32_t pS;          // pilot CTAs per query tile
+    int32_t G;           // pilot group maxima per query (groups of 32 references)
+    int32_t cprime;      // order statistic of the group maxima used as threshold
+    int32_t cap;         // list capacity per (query, split)
+    bool pilot;          // there are groups enough for the order statistic
+};
+DiffPlan diff_plan(int64_t n, int64_t m, int32_t d, int32_t c, int num_sms);
+cudaError_t launch_diff_pilot(const DiffPlan& p, const float* Q, int64_t n, const float* R, int64_t m,
+                              int32_t d, int32_t metric, uint32_t* gmax, cudaStream_t st, int* launches);
+// Also clears the two counters.
+cudaError_t launch_diff_threshold(const DiffPlan& p, const uint32_t* gmax, int64_t n, float* thr,
+                                  int32_t* count0, int32_t* count1, cudaStream_t st, int* launches);
+cudaError_t launch_diff_filter(const DiffPlan& p, const float* Q, int64_t n, const float* R, int64_t m,
+                               int32_t d, int32_t metric, const float* thr, uint64_t* lists,
+                               int32_t* counts, cudaStream_t st, int* launches);
 
 // The largest c launch_cc_select supports.
 int cc_max_candidates();

@@ -1003,39 +1003,18 @@ __global__ void prepare_kernel(const float* __restrict__ X, int64_t rows, int32_
 
 // One warp per query: the cprime-th largest group maximum of the pilot becomes
 // the query's threshold, written into its threshold words with a margin that
-// covers the rounding difference between the pilot and filter products.  The
-// maxima (order-mapped, 0 = no group) sit in registers, VPL per lane; the
+// covers the rounding difference between the pilot and filter products.
+//
+// order_statistic: the cprime-th largest of the G maxima of one query.  They
+// (order-mapped, 0 = no group) sit in registers, VPL per lane; the
 // order statistic is found bit by bit from the top (is the count of values
 // >= prefix|bit at least cprime?) down to bit 8.  Stopping there leaves a
 // value at most 2^8 order steps (2^-15 relative) below the exact one: a
 // slightly lower threshold, so never fewer passing references.
 //
-// Operand pairs (PREC = kPair): qscale[q] holds the query's squared norm n_q;
-// in its place goes the bound that certifies the query's answer.  With the
-// norm words slack of the reference folded in (pair_slack), every reference
-// has ||q - r||^2 >= bound - 2 acc, so those that fail the filter are at least
-// `bound` away.  A query whose norm is not finite or above 1e36 (where float32
-// squares overflow) gets -inf: it is never certified.
-template <int PREC, int VPL>
-__device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gmax, int64_t q,
-                                                int32_t G, int32_t cprime, int32_t d, int32_t kp,
-                                                void* __restrict__ Q_lp,
-                                                const uint32_t* __restrict__ rmax2,
-                                                float* __restrict__ qscale, int lane) {
-    const uint32_t* src = gmax + q * G;
-    // squared norm of the (low-precision) query row, for the hit-code scale
-    const size_t elt = (PREC == kTF32) ? 4 : 2;
-    void* row = static_cast<unsigned char*>(Q_lp) + static_cast<size_t>(q) * kp * elt;
-    float nq2 = 0.f;
-    if constexpr (PREC == kPair) {
-        nq2 = qscale[q];
-    } else {
-        for (int t = lane; t < d; t += 32) {
-            const float x = get<PREC>(row, t);
-            nq2 = fmaf(x, x, nq2);
-        }
-        for (int o = 16; o > 0; o >>= 1) nq2 += __shfl_xor_sync(0xffffffffu, nq2, o);
-    }
+template <int VPL>
+__device__ __forceinline__ uint32_t order_statistic(const uint32_t* __restrict__ src, int32_t G,
+                                                    int32_t cprime, int lane) {
     uint32_t v[VPL];
     uint32_t least = 0xffffffffu, most = 0u;
     int nvalid = 0;
@@ -1064,7 +1043,36 @@ __device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gma
         for (int i = 0; i < VPL; ++i) c += (v[i] >= cand) ? 1 : 0;
         if (__reduce_add_sync(0xffffffffu, c) >= cprime) prefix = cand;
     }
-    const uint32_t best = nvalid >= cprime ? prefix : least;   // fewer than cprime groups: the weakest
+    return nvalid >= cprime ? prefix : least;   // fewer than cprime groups: the weakest
+}
+
+// Operand pairs (PREC = kPair): qscale[q] holds the query's squared norm n_q;
+// in its place goes the bound that certifies the query's answer.  With the
+// norm words slack of the reference folded in (pair_slack), every reference
+// has ||q - r||^2 >= bound - 2 acc, so those that fail the filter are at least
+// `bound` away.  A query whose norm is not finite or above 1e36 (where float32
+// squares overflow) gets -inf: it is never certified.
+template <int PREC, int VPL>
+__device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gmax, int64_t q,
+                                                int32_t G, int32_t cprime, int32_t d, int32_t kp,
+                                                void* __restrict__ Q_lp,
+                                                const uint32_t* __restrict__ rmax2,
+                                                float* __restrict__ qscale, int lane) {
+    const uint32_t* src = gmax + q * G;
+    // squared norm of the (low-precision) query row, for the hit-code scale
+    const size_t elt = (PREC == kTF32) ? 4 : 2;
+    void* row = static_cast<unsigned char*>(Q_lp) + static_cast<size_t>(q) * kp * elt;
+    float nq2 = 0.f;
+    if constexpr (PREC == kPair) {
+        nq2 = qscale[q];
+    } else {
+        for (int t = lane; t < d; t += 32) {
+            const float x = get<PREC>(row, t);
+            nq2 = fmaf(x, x, nq2);
+        }
+        for (int o = 16; o > 0; o >>= 1) nq2 += __shfl_xor_sync(0xffffffffu, nq2, o);
+    }
+    const uint32_t best = order_statistic<VPL>(src, G, cprime, lane);
     const float t_acc = unord_f32(best);
     if constexpr (PREC == kPair) {
         const float tc = -t_acc + 1e-4f * fabsf(t_acc) + 1e-5f * nq2;
