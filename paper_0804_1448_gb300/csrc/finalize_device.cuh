@@ -704,59 +704,13 @@ __device__ __forceinline__ void queue_fallback(const FinalizeArgs& a, int64_t q,
     if (a.fallback_reason) atomicAdd(&a.fallback_reason[reason], 1ull);
 }
 
-// Query q, start to end, by one warp (lane = its lane): scratch is the warp's
-// shared memory (warp_scratch_bytes for these P, S, d and staging entries).
-// Every step is warp-synchronous; nothing waits on the rest of the CTA.
-// crow: the query's row of the candidate set (q unless the pass runs over a
-// queue).  CERT: hit lists of a float32 filter, whose answers are certified by
-// the lists' bound.
-template <int METRIC, int NV, int CERT = kNoCert>
-__device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, int64_t q,
-                               unsigned char* scratch, int lane, int64_t crow) {
+// The candidates' exact keys to the outputs: steps 2 to 5, by one warp.  w.keys
+// holds `pool` keys; cut is the certified list's (0 otherwise).
+template <int METRIC, int NV, int CERT>
+__device__ void finish_query(const FinalizeArgs& a, int Lcap, int64_t q, WarpScratch& w, int lane,
+                             int pool, float cut) {
     const int S = a.use_hits ? 1 : a.cand.S;
     const int d = a.d, k = a.k;
-    const int Lcap = prefix_cap(P, k);
-    const int se = a.use_hits ? stage_entries : 0;   // staging entries (hit lists only)
-    WarpScratch w = carve(scratch, P, Lcap, S, se);
-    // entries that fit keys[P] and the staging area behind it (contiguous)
-    const size_t union_bytes = prefix_bytes(Lcap) > static_cast<size_t>(se) * 8
-                                   ? prefix_bytes(Lcap) : static_cast<size_t>(se) * 8;
-    const int stage_all = static_cast<int>((align16(static_cast<size_t>(P) * 8) + union_bytes) / 8);
-    // the query row: its loads are issued before the hit-list sizes are read
-    const float* qg = a.Q + q * d;
-    float4 qv = make_float4(0.f, 0.f, 0.f, 0.f);
-    const bool qvec = NV > 0 && (reinterpret_cast<uintptr_t>(a.Q) & 15) == 0;
-    if (qvec) {
-        if (lane < (d >> 2)) qv = __ldg(reinterpret_cast<const float4*>(qg) + lane);
-    } else {
-        for (int t = lane; t < d; t += 32) w.qrow[t] = qg[t];
-    }
-    int total = 0, over = 0;
-    if (a.use_hits) hit_totals(a, q, lane, &total, &over);
-    if (qvec && lane < (d >> 2)) reinterpret_cast<float4*>(w.qrow)[lane] = qv;
-    for (int s = lane; s < S; s += 32) w.smax[s] = 0;
-    __syncwarp();
-
-    // 1. candidates with exact float32 keys
-    int pool;
-    float cut = 0.f;
-    if (!a.use_hits) {
-        pool = a.cand.S * a.cand.c;
-        gather_cand<METRIC, NV>(a, crow, w, lane);
-    } else {
-        if (over) pool = -2;
-        else if (total < a.hits.c && total < a.m) pool = -1;
-        else if (total <= kStage) pool = gather_hits_impl<METRIC, NV, 1, CERT>(a, q, P, w, lane, total, &cut);
-        else if (total <= stage_all)
-            pool = gather_hits_impl<METRIC, NV, 2, CERT>(a, q, P, w, lane, total, &cut);
-        else pool = gather_hits_impl<METRIC, NV, 0, CERT>(a, q, P, w, lane, total, &cut);
-        if (pool < 0) {
-            if (lane == 0) queue_fallback(a, q, -pool - 1);
-            return;
-        }
-    }
-    __syncwarp();
-
     // 2. ascending prefix by repeated minimum: the first k, continued through
     //    the near-tie run holding position k-1
     const float relf = a.relf;
@@ -985,6 +939,61 @@ __device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, 
     }
 }
 
+// Query q, start to end, by one warp (lane = its lane): scratch is the warp's
+// shared memory (warp_scratch_bytes for these P, S, d and staging entries).
+// Every step is warp-synchronous; nothing waits on the rest of the CTA.
+// crow: the query's row of the candidate set (q unless the pass runs over a
+// queue).  CERT: hit lists of a float32 filter, whose answers are certified by
+// the lists' bound.
+template <int METRIC, int NV, int CERT = kNoCert>
+__device__ void finalize_query(const FinalizeArgs& a, int P, int stage_entries, int64_t q,
+                               unsigned char* scratch, int lane, int64_t crow) {
+    const int S = a.use_hits ? 1 : a.cand.S;
+    const int d = a.d;
+    const int Lcap = prefix_cap(P, a.k);
+    const int se = a.use_hits ? stage_entries : 0;   // staging entries (hit lists only)
+    WarpScratch w = carve(scratch, P, Lcap, S, se);
+    // entries that fit keys[P] and the staging area behind it (contiguous)
+    const size_t union_bytes = prefix_bytes(Lcap) > static_cast<size_t>(se) * 8
+                                   ? prefix_bytes(Lcap) : static_cast<size_t>(se) * 8;
+    const int stage_all = static_cast<int>((align16(static_cast<size_t>(P) * 8) + union_bytes) / 8);
+    // the query row: its loads are issued before the hit-list sizes are read
+    const float* qg = a.Q + q * d;
+    float4 qv = make_float4(0.f, 0.f, 0.f, 0.f);
+    const bool qvec = NV > 0 && (reinterpret_cast<uintptr_t>(a.Q) & 15) == 0;
+    if (qvec) {
+        if (lane < (d >> 2)) qv = __ldg(reinterpret_cast<const float4*>(qg) + lane);
+    } else {
+        for (int t = lane; t < d; t += 32) w.qrow[t] = qg[t];
+    }
+    int total = 0, over = 0;
+    if (a.use_hits) hit_totals(a, q, lane, &total, &over);
+    if (qvec && lane < (d >> 2)) reinterpret_cast<float4*>(w.qrow)[lane] = qv;
+    for (int s = lane; s < S; s += 32) w.smax[s] = 0;
+    __syncwarp();
+
+    // 1. candidates with exact float32 keys
+    int pool;
+    float cut = 0.f;
+    if (!a.use_hits) {
+        pool = a.cand.S * a.cand.c;
+        gather_cand<METRIC, NV>(a, crow, w, lane);
+    } else {
+        if (over) pool = -2;
+        else if (total < a.hits.c && total < a.m) pool = -1;
+        else if (total <= kStage) pool = gather_hits_impl<METRIC, NV, 1, CERT>(a, q, P, w, lane, total, &cut);
+        else if (total <= stage_all)
+            pool = gather_hits_impl<METRIC, NV, 2, CERT>(a, q, P, w, lane, total, &cut);
+        else pool = gather_hits_impl<METRIC, NV, 0, CERT>(a, q, P, w, lane, total, &cut);
+        if (pool < 0) {
+            if (lane == 0) queue_fallback(a, q, -pool - 1);
+            return;
+        }
+    }
+    __syncwarp();
+    finish_query<METRIC, NV, CERT>(a, Lcap, q, w, lane, pool, cut);
+}
+
 template <int METRIC, int NV, int CERT>
 __global__ void __launch_bounds__(kFinThreads, 4)
 finalize_kernel(FinalizeArgs a, int P, int warps_per_block, int stage_entries) {
@@ -1008,6 +1017,175 @@ finalize_kernel(FinalizeArgs a, int P, int warps_per_block, int stage_entries) {
     const size_t per_warp =
         warp_scratch_bytes(P, prefix_cap(P, a.k), S, a.d, a.use_hits ? stage_entries : 0);
     finalize_query<METRIC, NV, CERT>(a, P, stage_entries, q, smem_raw + per_warp * warp, lane, row);
+}
+
+// Searches of few queries, hit lists: one CTA of kWideWarps warps per query.
+// A lone warp per query walks the lists, the cut and the re-rank one latency
+// after another on an idle GPU: 64 queries among 4 million points, 600 lists and
+// a thousand hits each, took it 102 us, and this one 20.  Here the warps share the lists, the
+// histogram and the candidates' distances; the first one finishes the query
+// (finish_query), and takes all of it when the lists outgrow the staging area.
+constexpr int kWideWarps = 8;
+constexpr int kWideThreads = 32 * kWideWarps;
+constexpr int kWideMaxQueries = 304;   // two CTAs per SM
+constexpr int kWideStage = 12288;
+
+struct WideShared {
+    int wsum[kWideWarps];
+    int cnt[kWideThreads];
+    float lo[kWideWarps], hi[kWideWarps];
+    int over, kept, cut1, cut2, before;
+};
+
+__device__ __forceinline__ float block_min(float v, float* slots, int warp, int lane) {
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if (lane == 0) slots[warp] = v;
+    __syncthreads();
+    v = slots[0];
+    for (int i = 1; i < kWideWarps; ++i) v = fminf(v, slots[i]);
+    return v;
+}
+
+template <int METRIC, int NV, int CERT>
+__global__ void __launch_bounds__(kWideThreads)
+finalize_wide_kernel(FinalizeArgs a, int P, int stage_entries) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ WideShared sh;
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    const int64_t q = blockIdx.x;
+    if (a.fb_done && blockIdx.x == 0 && tid < a.fb_slots) a.fb_done[tid] = 0;
+    const HitLists& hl = a.hits;
+    const int S = hl.S, cap = hl.cap, c = hl.c, d = a.d;
+    const int Lcap = prefix_cap(P, a.k);
+    WarpScratch w = carve(smem_raw, P, Lcap, 1, stage_entries);
+    const int32_t* cnts = hl.counts + q * static_cast<int64_t>(S);
+    const uint64_t* base = hl.keys + q * static_cast<int64_t>(S) * cap;
+    for (int t = tid; t < d; t += kWideThreads) w.qrow[t] = a.Q[q * d + t];
+    if (tid == 0) {
+        sh.over = 0;
+        sh.kept = 0;
+    }
+    __syncthreads();
+    // the lists, one after another into the staging area
+    int total = 0;
+    for (int s0 = 0; s0 < S; s0 += kWideThreads) {
+        const int raw = s0 + tid < S ? cnts[s0 + tid] : 0;
+        if (raw > cap) sh.over = 1;
+        const int mine = min(raw, cap);
+        int incl = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        __syncthreads();   // the last batch's counts and sums are read
+        if (lane == 31) sh.wsum[warp] = incl;
+        __syncthreads();
+        int at = total + incl - mine;
+        int sum = 0;
+        for (int x = 0; x < kWideWarps; ++x) {
+            if (x < warp) at += sh.wsum[x];
+            sum += sh.wsum[x];
+        }
+        if (total + sum <= stage_entries) {
+            if (S >= 64) {   // many short lists: one per thread
+                const uint64_t* sp = base + static_cast<int64_t>(s0 + tid) * cap;
+                for (int e = 0; e < mine; ++e) cp_async8(w.stage + at + e, sp + e);
+            } else {         // few long ones: one per warp
+                sh.cnt[tid] = at;
+                __syncthreads();
+                for (int s = warp; s < S; s += kWideWarps) {
+                    const int n_s = min(cnts[s], cap), o = sh.cnt[s];
+                    const uint64_t* sp = base + static_cast<int64_t>(s) * cap;
+                    for (int e = lane; e < n_s; e += 32) cp_async8(w.stage + o + e, sp + e);
+                }
+            }
+        }
+        total += sum;
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    if (sh.over || (total < c && total < a.m)) {
+        if (tid == 0) queue_fallback(a, q, sh.over ? 1 : 0);
+        return;
+    }
+    if (total > stage_entries) {
+        if (warp == 0) finalize_query<METRIC, NV, CERT>(a, P, stage_entries, q, smem_raw, lane, q);
+        return;
+    }
+    auto val = [&](int e) { return hit_val<CERT>(static_cast<uint32_t>(w.stage[e] >> 32)); };
+    float vmin = __int_as_float(0x7f800000), vneg = vmin;
+    for (int e = tid; e < total; e += kWideThreads) {
+        const float v = val(e);
+        vmin = fminf(vmin, v);
+        vneg = fminf(vneg, -v);
+    }
+    vmin = block_min(vmin, sh.lo, warp, lane);
+    const float vmax = -block_min(vneg, sh.hi, warp, lane);
+    const float range = vmax - vmin;
+    FastBin b1{vmin, range > 1e-30f ? (kBins - 0.51f) / range : 0.f};
+    int cut1 = kBins - 1, cut2 = kBins - 1;
+    Binning b2{0.f, 0.f};
+    if (total > c) {
+        if (tid < kBins) w.hist[tid] = 0;
+        __syncthreads();
+        for (int e = tid; e < total; e += kWideThreads) atomicAdd(&w.hist[b1.bin(val(e))], 1);
+        __syncthreads();
+        if (warp == 0) {
+            int cut, before;
+            cut_bin(w.hist, c, lane, &cut, &before);
+            if (lane == 0) {
+                sh.cut1 = cut;
+                sh.before = before;
+            }
+        }
+        __syncthreads();
+        cut1 = sh.cut1;
+        const int before = sh.before, in_bin = w.hist[cut1];
+        __syncthreads();
+        if (before + in_bin > P && b1.inv > 0.f) {   // refine the cut bin once
+            b2.lo = vmin + (cut1 - 0.5f) / b1.inv;
+            b2.inv = b1.inv * kBins;
+            if (tid < kBins) w.hist[tid] = 0;
+            __syncthreads();
+            for (int e = tid; e < total; e += kWideThreads) {
+                const float v = val(e);
+                if (b1.bin(v) == cut1) atomicAdd(&w.hist[b2.bin(v)], 1);
+            }
+            __syncthreads();
+            if (warp == 0) {
+                int cut, unused;
+                cut_bin(w.hist, c - before, lane, &cut, &unused);
+                if (lane == 0) sh.cut2 = cut;
+            }
+            __syncthreads();
+            cut2 = sh.cut2;
+        }
+    }
+    float cut = CERT == kCertDiff ? __int_as_float(0x7f800000) : 0.f;
+    for (int e = tid; e < total; e += kWideThreads) {
+        const uint64_t key = w.stage[e];
+        const float v = hit_val<CERT>(static_cast<uint32_t>(key >> 32));
+        const int bb = b1.bin(v);
+        if (bb < cut1 || (bb == cut1 && (b2.inv == 0.f || b2.bin(v) <= cut2))) {
+            const int pos = atomicAdd(&sh.kept, 1);
+            if (pos < P) w.keys[pos] = key_idx(key);
+        } else {
+            cut = fminf(cut, v);
+        }
+    }
+    if (CERT) cut = block_min(cut, sh.lo, warp, lane);
+    __syncthreads();
+    const int kept = sh.kept;
+    if (kept > P) {
+        if (tid == 0) queue_fallback(a, q, 2);
+        return;
+    }
+    const int share = (kept + kWideWarps - 1) / kWideWarps;
+    const int first = min(kept, warp * share);
+    exact_keys<METRIC, NV>(w.keys + first, min(kept - first, share), a.R, d, w.qrow, lane);
+    __syncthreads();
+    if (warp == 0) finish_query<METRIC, NV, CERT>(a, Lcap, q, w, lane, kept, cut);
 }
 
 // ---------------------------------------------------------------------------

@@ -1,6 +1,8 @@
 // knn_finalize.cu -- host side of the finalize and exact-fallback stages
 // (launch shapes, launchers) and the self-join row pass.  The device code, and
 // the description of the stages, is in finalize_device.cuh.
+#include <algorithm>
+
 #include "finalize_device.cuh"
 
 namespace knn {
@@ -42,6 +44,25 @@ cudaError_t launch_finalize_nv(const FinalizeArgs& a, int P, int wpb, int se, si
     return cudaGetLastError();
 }
 
+template <int METRIC, int NV, int CERT>
+cudaError_t launch_wide_nv(const FinalizeArgs& a, int P, int se, size_t smem, cudaStream_t st) {
+    cudaError_t err = allow_smem<finalize_wide_kernel<METRIC, NV, CERT>>(smem);
+    if (err != cudaSuccess) return err;
+    finalize_wide_kernel<METRIC, NV, CERT><<<static_cast<unsigned>(a.n), kWideThreads, smem, st>>>(a, P, se);
+    return cudaGetLastError();
+}
+
+template <int METRIC, int CERT>
+cudaError_t launch_wide(const FinalizeArgs& a, int nv, int P, int se, size_t smem, cudaStream_t st) {
+    switch (nv) {
+        case 1: return launch_wide_nv<METRIC, 1, CERT>(a, P, se, smem, st);
+        case 2: return launch_wide_nv<METRIC, 2, CERT>(a, P, se, smem, st);
+        case 3: return launch_wide_nv<METRIC, 3, CERT>(a, P, se, smem, st);
+        case 4: return launch_wide_nv<METRIC, 4, CERT>(a, P, se, smem, st);
+        default: return launch_wide_nv<METRIC, 0, CERT>(a, P, se, smem, st);
+    }
+}
+
 template <int METRIC, int CERT = kNoCert>
 cudaError_t launch_finalize_m(const FinalizeArgs& a, int nv, int P, int wpb, int se, size_t smem,
                               unsigned grid, cudaStream_t st) {
@@ -62,14 +83,7 @@ cudaError_t launch_finalize(const FinalizeArgs& a_in, cudaStream_t st, int* laun
     int P = a.use_hits ? 2 * a.hits.c + 32 : a.cand.S * a.cand.c;
     P = (P + 3) & ~3;
     if (P > kMaxPool) return cudaErrorInvalidValue;
-    // hit-list staging: kStage entries; when the queries do not fill the GPU
-    // anyway, room for every list entry a query can have (up to 12288), so
-    // long lists are still read from shared memory
-    int se = a.use_hits ? kStage : 0;
-    if (a.use_hits && a.n <= 256) {
-        const int64_t all = static_cast<int64_t>(a.hits.S) * a.hits.cap;
-        se = static_cast<int>(all < kStage ? kStage : (all > 12288 ? 12288 : all));
-    }
+    const int se = a.use_hits ? kStage : 0;   // hit-list staging entries
     const size_t per_warp = warp_scratch_bytes(P, prefix_cap(P, a.k), a.use_hits ? 1 : a.cand.S,
                                                a.d, se);
     // up to eight warps per block and four blocks per SM when the scratch allows
@@ -84,6 +98,18 @@ cudaError_t launch_finalize(const FinalizeArgs& a_in, cudaStream_t st, int* laun
         ((reinterpret_cast<uintptr_t>(a.R) | reinterpret_cast<uintptr_t>(a.Q)) & 15) == 0;
     const int nv = (aligned && (a.d & 3) == 0 && a.d <= 128) ? (a.d + 31) / 32 : 0;
     if (launches) ++*launches;
+    if (a.use_hits && a.n <= kWideMaxQueries) {
+        // one CTA per query, staging room for every list entry (up to kWideStage)
+        const int64_t all = static_cast<int64_t>(a.hits.S) * a.hits.cap;
+        const int wide = static_cast<int>(std::min<int64_t>(std::max<int64_t>(all, kStage), kWideStage));
+        const size_t ws = warp_scratch_bytes(P, prefix_cap(P, a.k), 1, a.d, wide);
+        if (ws + sizeof(WideShared) <= 200 * 1024) {
+            if (!a.hits.bound) return launch_wide<kL2, kNoCert>(a, nv, P, wide, ws, st);
+            if (a.metric == kL2) return launch_wide<kL2, kCertPair>(a, nv, P, wide, ws, st);
+            if (a.metric == kL1) return launch_wide<kL1, kCertDiff>(a, nv, P, wide, ws, st);
+            return launch_wide<kLinf, kCertDiff>(a, nv, P, wide, ws, st);
+        }
+    }
     if (a.use_hits && a.hits.bound) {
         if (a.metric == kL2) return launch_finalize_m<kL2, kCertPair>(a, nv, P, wpb, se, smem, grid, st);
         if (a.metric == kL1) return launch_finalize_m<kL1, kCertDiff>(a, nv, P, wpb, se, smem, grid, st);
