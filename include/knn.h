@@ -336,7 +336,9 @@ knn_status knn_create_shared(knn_handle* out, knn_handle src, const knn_options*
  * io_on_device, ...) needs with h's current reference set and precision
  * (written to *bytes; 0 for n = 0).  Nothing is allocated or launched.  With
  * knn_reserve, this lets a caller admit work by memory and keep allocation
- * out of the search path.
+ * out of the search path.  (A float32 Euclidean search of a large set includes
+ * a copy of the set split into bf16 pairs, about as large as the set; under a
+ * workspace_limit too small for it, it plans without.)
  * Errors: as knn_search's argument checks (KNN_ERR_INVALID, KNN_ERR_NOREF,
  * KNN_ERR_UNSUPPORTED); KNN_ERR_INVALID when bytes is NULL.
  */

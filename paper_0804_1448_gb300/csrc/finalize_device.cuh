@@ -998,6 +998,7 @@ template <int METRIC, int NV, int CERT>
 __global__ void __launch_bounds__(kFinThreads, 4)
 finalize_kernel(FinalizeArgs a, int P, int warps_per_block, int stage_entries) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_begin();
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int64_t row = static_cast<int64_t>(blockIdx.x) * warps_per_block + warp;
     int64_t q = row;
@@ -1052,6 +1053,7 @@ __global__ void __launch_bounds__(kWideThreads)
 finalize_wide_kernel(FinalizeArgs a, int P, int stage_entries) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ WideShared sh;
+    chain_begin();
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int64_t q = blockIdx.x;
     if (a.fb_done && blockIdx.x == 0 && tid < a.fb_slots) a.fb_done[tid] = 0;
@@ -1494,6 +1496,7 @@ fallback_kernel(FinalizeArgs a, double* __restrict__ scratch, int32_t* __restric
     __shared__ FbShared<kFbThreads> sh;
     __shared__ int last;
     extern __shared__ __align__(16) unsigned char fb_dyn[];
+    chain_begin();
     const FbDyn f = fb_dyn_carve(fb_dyn);
     const int tid = threadIdx.x;
     const int count = *a.fallback_count;

@@ -511,7 +511,8 @@ struct RefView {
 knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, const float* Qd,
                           int64_t n, int32_t k, knn_metric metric, float* dd, int32_t* id,
                           unsigned char* ws, int32_t* fallback_count, cudaStream_t st, int* l,
-                          bool stages, float* Q_copy = nullptr, cudaEvent_t prep_done = nullptr) {
+                          bool stages, bool chain, float* Q_copy = nullptr,
+                          cudaEvent_t prep_done = nullptr) {
     const int64_t m = rv.m;
     const int32_t d = rv.d;
     const int S = sp.S, c = sp.c;
@@ -524,11 +525,10 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
     if (sp.filtered()) {
         queue.count = reinterpret_cast<int32_t*>(ws + sp.off_queue);
         queue.list = queue.count + 1;
-    } else {
-        KNN_CUDA(h, cudaMemsetAsync(fallback_count, 0, sizeof(int32_t), st));
     }
     if (sp.tensor || sp.pair) {
-        const TcPlan& plan = sp.plan;
+        TcPlan plan = sp.plan;
+        plan.chain = chain;
         const int prec = sp.prec;
         const void* R_lp = sp.pair ? ws + sp.off_rl : rv.R_lp;
         const int32_t kp = sp.pair ? sp.kp : rv.kp;
@@ -545,7 +545,8 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
             KNN_CUDA(h, launch_prepare_pair(rv.R, m, Qd, n, d, kp, ws + sp.off_rl, Ql, qs.qscale,
                                             queue.count, fallback_count, st, l));
         else
-            KNN_CUDA(h, launch_prepare_query(Qd, n, d, kp, prec, Ql, qs_prep, Q_copy, st, l));
+            KNN_CUDA(h, launch_prepare_query(Qd, n, d, kp, prec, Ql, qs_prep, Q_copy, fallback_count,
+                                             st, l));
         if (Q_copy) Qd = Q_copy;
         mark("prepare_q");
         if (prep_done) KNN_CUDA(h, cudaEventRecord(prep_done, st));
@@ -570,7 +571,8 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
         fa.cand.S = 1;
         fa.cand.c = c;
     } else if (sp.diff) {
-        const DiffPlan& dp = sp.dplan;
+        DiffPlan dp = sp.dplan;
+        dp.chain = chain;
         uint32_t* gmax = reinterpret_cast<uint32_t*>(ws + sp.off_gmax);
         float* thr = reinterpret_cast<float*>(ws + sp.off_qs);
         uint64_t* lists = reinterpret_cast<uint64_t*>(ws + sp.off_lists);
@@ -592,13 +594,14 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
         fa.cand.S = 1;
         fa.cand.c = c;
     } else {
-        CandidateSet cs;
+        CandidateSet cs{};
         cs.keys = reinterpret_cast<uint64_t*>(ws + sp.off_cand);
         cs.n = n;
         cs.S = S;
         cs.c = c;
         cs.chunk = sp.chunk;
         cs.exact = 1;
+        cs.clear = fallback_count;
         if (sp.small) {
             KNN_CUDA(h, launch_small_select(Qd, n, rv.R, m, d, metric, sp.c_need, cs, st, l));
             mark("small_select");
@@ -625,6 +628,7 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
     fa.fallback_reason = ctr->fallback_reason;
     fa.fb_done = reinterpret_cast<int32_t*>(ws + sp.off_fbdone);
     fa.fb_slots = static_cast<int32_t>(sp.fb_grid);
+    fa.chain = chain ? 1 : 0;
     if (sp.filtered()) {
         // the filter's answers; the queries it cannot certify go through the
         // CUDA-core select (a few: straight to the exact fallback)
@@ -635,13 +639,14 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
         fp.fb_done = nullptr;
         KNN_CUDA(h, launch_finalize(fp, st, l));
         mark("finalize");
-        CandidateSet cs;
+        CandidateSet cs{};
         cs.keys = reinterpret_cast<uint64_t*>(ws + sp.off_cand);
         cs.n = n;
         cs.S = S;
         cs.c = c;
         cs.chunk = sp.chunk;
         cs.exact = 1;
+        cs.chain = chain ? 1 : 0;
         KNN_CUDA(h, launch_cc_select(Qd, n, rv.R, m, d, metric, cs, st, l, queue));
         fa.use_hits = 0;
         fa.hits = HitLists{};
@@ -765,7 +770,7 @@ knn_status enqueue_instance(knn_ctx* h, const knn_instance& x, const BatchPlan& 
     }
     return enqueue_search(h, sp, rv, x.Q, x.n, x.k, static_cast<knn_metric>(x.metric), x.dist_out,
                           x.idx_out, ws + bp.base[i], reinterpret_cast<int32_t*>(ws + bp.fbc[i]),
-                          st, l, false);
+                          st, l, false, false);
 }
 
 // The side streams and events of a host-buffer search run in parts.
@@ -1287,7 +1292,7 @@ knn_status knn_search(knn_handle h, const float* Q, int64_t n, int32_t d, int32_
             unsigned char* wj = ws + poff[j];
             int32_t* fc = j == 0 ? &ctr->fallback_count : &ctr->fallback_part[j - 1];
             s = enqueue_search(h, pp[j], rv, Q + pb[j] * d, pb[j + 1] - pb[j], k, metric,
-                               dist_out + pb[j] * k, idx_out + pb[j] * k, wj, fc, sj, &l, false,
+                               dist_out + pb[j] * k, idx_out + pb[j] * k, wj, fc, sj, &l, false, false,
                                reinterpret_cast<float*>(wj + pp[j].off_q),
                                j + 1 < parts ? h->pipe_prep[j] : nullptr);
             if (s != KNN_OK) return s;
@@ -1298,7 +1303,7 @@ knn_status knn_search(knn_handle h, const float* Q, int64_t n, int32_t d, int32_
         }
     } else {
         s = enqueue_search(h, sp, rv, Qd, n, k, metric, dd, id, ws, &ctr->fallback_count, st, &l,
-                           true, q_copy);
+                           true, io_on_device != 0, q_copy);
         if (s != KNN_OK) return s;
     }
     h->launches += l;
@@ -1525,7 +1530,7 @@ knn_status knn_search_self(knn_handle h, int32_t k, knn_metric metric, float* di
     h->nstages = 0;
     RefView rv{rs.R, rs.m, rs.d, rs.R_lp, rs.kp, rs.rmax2};
     s = enqueue_search(h, sp, rv, rs.R, n, k + 1, metric, dtmp, itmp, ws, &h->counters->fallback_count,
-                       st, &l, false);
+                       st, &l, false, true);
     if (s != KNN_OK) return s;
     KNN_CUDA(h, launch_drop_self(dtmp, itmp, n, k, dist_out, idx_out, st, &l));
     h->launches += l;

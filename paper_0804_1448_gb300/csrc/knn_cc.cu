@@ -156,6 +156,8 @@ template <int METRIC, int ROWS, bool QUEUED>
 __global__ void __launch_bounds__(kThreads, CCShape<ROWS>::MINB)
 cc_select_kernel(const float* __restrict__ Q, int64_t n, const float* __restrict__ R,
                  int64_t m, int32_t d, CandidateSet cand, QueryQueue from) {
+    chain_begin();
+    if (cand.clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *cand.clear = 0;
     if constexpr (QUEUED) {
         const int count = *from.count;
         if (count <= kDirectQueue || static_cast<int64_t>(blockIdx.x) * ROWS >= count) return;
@@ -442,7 +444,8 @@ cudaError_t launch_rows(const float* Q, int64_t n, const float* R, int64_t m, in
     cudaError_t err = allow_smem<cc_select_kernel<METRIC, ROWS, QUEUED>>(smem);
     if (err != cudaSuccess) return err;
     dim3 grid(static_cast<unsigned>((n + ROWS - 1) / ROWS), static_cast<unsigned>(cand.S));
-    kern<<<grid, kThreads, smem, st>>>(Q, n, R, m, d, cand, from);
+    if (QUEUED) return launch_chained(cand.chain != 0, kern, grid, dim3(kThreads), smem, st, Q, n, R, m, d, cand, from);
+    kern<<<grid, kThreads, smem, st>>>(Q, n, R, m, d, cand, from);   // a search's first kernel
     return cudaGetLastError();
 }
 

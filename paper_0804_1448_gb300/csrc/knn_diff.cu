@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(kThreads, Shape<ROWS>::MINB) diff_kernel(DiffA
     constexpr int RPT = kTM * kDK / kThreads;
     constexpr float kInf = __builtin_huge_valf();
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     const int d = a.d, dp = padded_d(d);
     float* Qs = sm;                                    // [dp][QST]
     float* Rs = Qs + static_cast<size_t>(dp) * QST;    // [kRing][kDK][kRST]
@@ -306,6 +307,7 @@ template <int VPL>
 __global__ void diff_threshold_kernel(const uint32_t* __restrict__ gmax, int64_t n, int32_t G,
                                       int32_t cprime, float* __restrict__ thr,
                                       int32_t* __restrict__ count0, int32_t* __restrict__ count1) {
+    chain_begin();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *count0 = 0;
         *count1 = 0;
@@ -318,22 +320,22 @@ __global__ void diff_threshold_kernel(const uint32_t* __restrict__ gmax, int64_t
 }
 
 template <int METRIC, int ROWS>
-cudaError_t launch_shape(const DiffArgs& a, bool pilot, cudaStream_t st) {
+cudaError_t launch_shape(const DiffArgs& a, bool pilot, bool chain, cudaStream_t st) {
     const size_t smem = smem_bytes<ROWS>(a.d);
     const dim3 grid(static_cast<unsigned>((a.n + ROWS - 1) / ROWS), static_cast<unsigned>(a.S));
     cudaError_t err = pilot ? allow_smem<diff_kernel<METRIC, ROWS, true>>(smem)
                             : allow_smem<diff_kernel<METRIC, ROWS, false>>(smem);
     if (err != cudaSuccess) return err;
-    if (pilot) diff_kernel<METRIC, ROWS, true><<<grid, kThreads, smem, st>>>(a);
-    else diff_kernel<METRIC, ROWS, false><<<grid, kThreads, smem, st>>>(a);
+    if (!pilot) return launch_chained(chain, diff_kernel<METRIC, ROWS, false>, grid, dim3(kThreads), smem, st, a);
+    diff_kernel<METRIC, ROWS, true><<<grid, kThreads, smem, st>>>(a);   // a search's first kernel
     return cudaGetLastError();
 }
 
 template <int METRIC>
-cudaError_t launch_metric(const DiffArgs& a, int rows, bool pilot, cudaStream_t st) {
-    if (rows == 128) return launch_shape<METRIC, 128>(a, pilot, st);
-    if (rows == 64) return launch_shape<METRIC, 64>(a, pilot, st);
-    return launch_shape<METRIC, 16>(a, pilot, st);
+cudaError_t launch_metric(const DiffArgs& a, int rows, bool pilot, bool chain, cudaStream_t st) {
+    if (rows == 128) return launch_shape<METRIC, 128>(a, pilot, chain, st);
+    if (rows == 64) return launch_shape<METRIC, 64>(a, pilot, chain, st);
+    return launch_shape<METRIC, 16>(a, pilot, chain, st);
 }
 
 DiffArgs base_args(const DiffPlan& p, const float* Q, int64_t n, const float* R, int64_t m, int32_t d) {
@@ -416,7 +418,7 @@ cudaError_t launch_diff_pilot(const DiffPlan& p, const float* Q, int64_t n, cons
     a.S = p.pS;
     a.gmax = gmax;
     if (launches) ++*launches;
-    return metric == kL1 ? launch_metric<kL1>(a, p.rows, true, st) : launch_metric<kLinf>(a, p.rows, true, st);
+    return metric == kL1 ? launch_metric<kL1>(a, p.rows, true, p.chain, st) : launch_metric<kLinf>(a, p.rows, true, p.chain, st);
 }
 
 cudaError_t launch_diff_threshold(const DiffPlan& p, const uint32_t* gmax, int64_t n, float* thr,
@@ -424,11 +426,11 @@ cudaError_t launch_diff_threshold(const DiffPlan& p, const uint32_t* gmax, int64
     const unsigned grid = static_cast<unsigned>((n + 7) / 8);
     const int vpl = (p.G + 31) / 32;
     if (launches) ++*launches;
-    if (vpl <= 4) diff_threshold_kernel<4><<<grid, 256, 0, st>>>(gmax, n, p.G, p.cprime, thr, count0, count1);
-    else if (vpl <= 16) diff_threshold_kernel<16><<<grid, 256, 0, st>>>(gmax, n, p.G, p.cprime, thr, count0, count1);
-    else if (vpl <= 64) diff_threshold_kernel<64><<<grid, 256, 0, st>>>(gmax, n, p.G, p.cprime, thr, count0, count1);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    if (vpl > 64) return cudaErrorInvalidValue;
+    return launch_chained(p.chain, vpl <= 4    ? diff_threshold_kernel<4>
+                          : vpl <= 16 ? diff_threshold_kernel<16>
+                                      : diff_threshold_kernel<64>,
+                          dim3(grid), dim3(256), 0, st, gmax, n, p.G, p.cprime, thr, count0, count1);
 }
 
 cudaError_t launch_diff_filter(const DiffPlan& p, const float* Q, int64_t n, const float* R, int64_t m,
@@ -439,7 +441,7 @@ cudaError_t launch_diff_filter(const DiffPlan& p, const float* Q, int64_t n, con
     a.lists = lists;
     a.counts = counts;
     if (launches) ++*launches;
-    return metric == kL1 ? launch_metric<kL1>(a, p.rows, false, st) : launch_metric<kLinf>(a, p.rows, false, st);
+    return metric == kL1 ? launch_metric<kL1>(a, p.rows, false, p.chain, st) : launch_metric<kLinf>(a, p.rows, false, p.chain, st);
 }
 
 }  // namespace knn

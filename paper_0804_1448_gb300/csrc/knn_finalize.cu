@@ -12,6 +12,7 @@ namespace knn {
 __global__ void drop_self_kernel(const float* __restrict__ din, const int32_t* __restrict__ iin,
                                  int64_t n, int32_t k, float* __restrict__ dout,
                                  int32_t* __restrict__ iout) {
+    chain_begin();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float* dr = din + i * (k + 1);
@@ -29,8 +30,7 @@ cudaError_t launch_drop_self(const float* din, const int32_t* iin, int64_t n, in
                              int32_t* iout, cudaStream_t st, int* launches) {
     const unsigned grid = static_cast<unsigned>((n + 255) / 256);
     if (launches) ++*launches;
-    drop_self_kernel<<<grid, 256, 0, st>>>(din, iin, n, k, dout, iout);
-    return cudaGetLastError();
+    return launch_chained(true, drop_self_kernel, dim3(grid), dim3(256), 0, st, din, iin, n, k, dout, iout);
 }
 
 int finalize_max_pool() { return kMaxPool; }
@@ -40,16 +40,16 @@ cudaError_t launch_finalize_nv(const FinalizeArgs& a, int P, int wpb, int se, si
                                unsigned grid, cudaStream_t st) {
     cudaError_t err = allow_smem<finalize_kernel<METRIC, NV, CERT>>(smem);
     if (err != cudaSuccess) return err;
-    finalize_kernel<METRIC, NV, CERT><<<grid, wpb * 32, smem, st>>>(a, P, wpb, se);
-    return cudaGetLastError();
+    return launch_chained(a.chain != 0, finalize_kernel<METRIC, NV, CERT>, dim3(grid), dim3(wpb * 32), smem, st, a, P,
+                          wpb, se);
 }
 
 template <int METRIC, int NV, int CERT>
 cudaError_t launch_wide_nv(const FinalizeArgs& a, int P, int se, size_t smem, cudaStream_t st) {
     cudaError_t err = allow_smem<finalize_wide_kernel<METRIC, NV, CERT>>(smem);
     if (err != cudaSuccess) return err;
-    finalize_wide_kernel<METRIC, NV, CERT><<<static_cast<unsigned>(a.n), kWideThreads, smem, st>>>(a, P, se);
-    return cudaGetLastError();
+    return launch_chained(a.chain != 0, finalize_wide_kernel<METRIC, NV, CERT>, dim3(static_cast<unsigned>(a.n)),
+                          dim3(kWideThreads), smem, st, a, P, se);
 }
 
 template <int METRIC, int CERT>
@@ -129,9 +129,8 @@ cudaError_t launch_fallback_m(const FinalizeArgs& a, double* scratch, int32_t sl
     // slot serves every queued query with one CTA)
     const int32_t spread = slots >= 2 ? slots / 2 : 0;
     const unsigned chunks = spread > 0 ? static_cast<unsigned>((a.m + kFbChunk - 1) / kFbChunk) : 1u;
-    fallback_kernel<METRIC><<<dim3(chunks, static_cast<unsigned>(slots)), kFbThreads, smem, st>>>(
-        a, scratch, done, spread);
-    return cudaGetLastError();
+    return launch_chained(a.chain != 0, fallback_kernel<METRIC>, dim3(chunks, static_cast<unsigned>(slots)),
+                          dim3(kFbThreads), smem, st, a, scratch, done, spread);
 }
 
 cudaError_t launch_fallback(const FinalizeArgs& a, double* scratch, int32_t slots, int32_t* done,

@@ -120,7 +120,7 @@ extern "C" knn_status knn_search_static(const float* R, int64_t m, const float* 
         (void)cudaGetLastError();
         return KNN_ERR_CUDA;
     }
-    CandidateSet cs;
+    CandidateSet cs{};
     cs.keys = reinterpret_cast<uint64_t*>(base + off_cand);
     cs.n = n;
     cs.S = S;

@@ -110,6 +110,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 small_select_kernel(const float* __restrict__ Q, int64_t n, const float* __restrict__ R,
                     int32_t m, int32_t d, int32_t c_need, CandidateSet cand) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
+    if (cand.clear && blockIdx.x == 0 && threadIdx.x == 0) *cand.clear = 0;
     const int pq = (d + kChunk - 1) / kChunk * kChunk;   // query pitch: whole chunks, zero padded
     float* Qw = sm;                                       // [kWarps][pq]
     float* Dw = Qw + kWarps * pq;                         // [kWarps][m]

@@ -62,8 +62,7 @@ cudaError_t launch_kernel(const TcPlan& p, const CUtensorMap& mq, const CUtensor
     cudaError_t err = allow_smem<tc_kernel<PREC, PILOT, KBT, EPI>>(smem);
     if (err != cudaSuccess) return err;
     dim3 grid(static_cast<unsigned>((a.n + kBlockM - 1) / kBlockM), static_cast<unsigned>(a.S));
-    kern<<<grid, kTcThreads, smem, st>>>(mq, mr, a);
-    return cudaGetLastError();
+    return launch_chained(p.chain, kern, grid, dim3(kTcThreads), smem, st, mq, mr, a);
 }
 
 template <int PREC, bool PILOT>
@@ -311,10 +310,10 @@ cudaError_t launch_prepare_ref(const float* R, int64_t m, int32_t d, int32_t kp,
     const unsigned grid = static_cast<unsigned>((warps * 32 + 255) / 256);
     if (prec == kBF16)
         prepare_kernel<kBF16, true><<<grid, 256, 0, st>>>(R, m, d, kp, R_lp, norms, rmax2, nullptr,
-                                                           nullptr);
+                                                           nullptr, nullptr);
     else
         prepare_kernel<kTF32, true><<<grid, 256, 0, st>>>(R, m, d, kp, R_lp, norms, rmax2, nullptr,
-                                                           nullptr);
+                                                           nullptr, nullptr);
     if (launches) ++*launches;
     return cudaGetLastError();
 }
@@ -334,18 +333,18 @@ cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* Q, int64
 }
 
 cudaError_t launch_prepare_query(const float* Q, int64_t n, int32_t d, int32_t kp, int prec,
-                                 void* Q_lp, const HitScale& qs, float* Q_copy, cudaStream_t st,
-                                 int* launches) {
+                                 void* Q_lp, const HitScale& qs, float* Q_copy, int32_t* clear,
+                                 cudaStream_t st, int* launches) {
     const int64_t warps = (n + kPrepRowsPerWarp - 1) / kPrepRowsPerWarp;
     const unsigned grid = static_cast<unsigned>((warps * 32 + 255) / 256);
     if (prec == kBF16)
         prepare_kernel<kBF16, false><<<grid, 256, 0, st>>>(Q, n, d, kp, Q_lp, nullptr,
                                                             const_cast<uint32_t*>(qs.rmax2), qs.qscale,
-                                                            Q_copy);
+                                                            Q_copy, clear);
     else
         prepare_kernel<kTF32, false><<<grid, 256, 0, st>>>(Q, n, d, kp, Q_lp, nullptr,
                                                             const_cast<uint32_t*>(qs.rmax2), qs.qscale,
-                                                            Q_copy);
+                                                            Q_copy, clear);
     if (launches) ++*launches;
     return cudaGetLastError();
 }
@@ -367,8 +366,8 @@ void launch_threshold_vpl(const TcPlan& p, const uint32_t* gmax, int64_t n, int3
                           void* Q_lp, const HitScale& qs, cudaStream_t st) {
     constexpr int wpb = 8;
     const unsigned grid = static_cast<unsigned>((n + wpb - 1) / wpb);
-    threshold_kernel<PREC, VPL><<<grid, wpb * 32, 0, st>>>(gmax, n, p.G, p.cprime, d, kp, Q_lp,
-                                                          qs.rmax2, qs.qscale);
+    (void)launch_chained(p.chain, threshold_kernel<PREC, VPL>, dim3(grid), dim3(wpb * 32), 0, st, gmax, n, p.G,
+                         p.cprime, d, kp, Q_lp, qs.rmax2, qs.qscale);
 }
 
 template <int PREC>

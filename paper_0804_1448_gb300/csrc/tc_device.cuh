@@ -638,6 +638,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_r,
           TcArgs a) {
     extern __shared__ unsigned char smem_raw[];
+    chain_begin();
     tc_run<PREC, PILOT, KBT, EPI, false>(&tmap_q, &tmap_r, a, blockIdx.x, blockIdx.y, smem_raw, 0u);
 }
 
@@ -738,6 +739,7 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
                                     uint32_t* __restrict__ R_lp, uint32_t* __restrict__ Q_lp,
                                     float* __restrict__ qnorm, int64_t ref_warps,
                                     int32_t* __restrict__ count0, int32_t* __restrict__ count1) {
+    chain_begin();
     constexpr int RW = kPairRows, NJ = kPairMaxD / 64;
     const int lane = threadIdx.x % 32;
     int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) / 32;
@@ -936,7 +938,9 @@ template <int PREC, bool REF>
 __global__ void prepare_kernel(const float* __restrict__ X, int64_t rows, int32_t d, int32_t kp,
                                void* __restrict__ out, float* __restrict__ norms,
                                uint32_t* __restrict__ rmax2, float* __restrict__ qscale,
-                               float* __restrict__ xcopy) {
+                               float* __restrict__ xcopy, int32_t* __restrict__ clear) {
+    chain_begin();
+    if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
     constexpr int RW = kPrepRowsPerWarp;
     const int lane = threadIdx.x % 32;
     const int64_t r0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * RW;
@@ -1107,6 +1111,7 @@ template <int PREC, int VPL>
 __global__ void threshold_kernel(const uint32_t* __restrict__ gmax, int64_t n, int32_t G,
                                  int32_t cprime, int32_t d, int32_t kp, void* __restrict__ Q_lp,
                                  const uint32_t* __restrict__ rmax2, float* __restrict__ qscale) {
+    chain_begin();
     const int64_t q = static_cast<int64_t>(blockIdx.x) * (blockDim.x / 32) + threadIdx.x / 32;
     if (q >= n) return;
     threshold_query<PREC, VPL>(gmax, q, G, cprime, d, kp, Q_lp, rmax2, qscale, threadIdx.x % 32);
