@@ -503,8 +503,8 @@ cudaError_t persist_build(const std::vector<PersistInst>& in, const PersistPlan&
         int vpl = 1;
         while (vpl * 32 < p.G) vpl *= 2;
         I.vpl = vpl;
-        if (!tc_make_map(&I.mq, I.Q_lp, x.n, pi.kp, prec, 128, 0) ||
-            !tc_make_map(&I.mr, I.R_lp, x.m, pi.kp, prec, p.rb, p.kbs))
+        if (!tc_make_map(&I.mq, I.Q_lp, x.n, pi.kp, prec, 128) ||
+            !tc_make_map(&I.mr, I.R_lp, x.m, pi.kp, prec, p.rb))
             return cudaErrorInvalidValue;
         TcArgs a{};
         a.n = x.n;

@@ -337,7 +337,7 @@ struct SearchPlan {
 // the faster form at every size above the small-set select's: one query among
 // 5000 references, d = 8, 52 us against 97 us with the CUDA-core select; 64
 // among 2 million, d = 96, 0.80 ms against 1.96; 4000 among 100000, d = 128,
-// 0.44 ms against 3.90; n = m = 38400, d = 96, 1.08 ms against 8.57.
+// 0.44 ms against 3.90; n = m = 38400, d = 96, 0.86 ms against 8.57.
 bool plan_pair(int64_t n, int64_t m, int32_t d, int32_t c, int sm_share, SearchPlan* p) {
     if (!pair_rows_fit(d) || 2 * c + 32 > finalize_max_pool()) return false;
     const int kp = tc_padded_dim(d, kPair);

@@ -292,13 +292,13 @@ enum LowPrecision : int { kTF32 = 1, kBF16 = 2, kPair = 3 };
 
 // Row length (elements) of the low-precision operand copies: d coordinates,
 // four augmentation words (norm halves, threshold halves), zero padded to a
-// whole number of 128-byte K blocks.
+// whole number of 32-byte MMA K steps.
 int tc_padded_dim(int32_t d, int prec);
 
 // Launch plan of the pilot and filter passes for one search.
 struct TcPlan {
     int32_t mt;          // 128-query tiles per CTA (1)
-    int32_t kb;          // 128-byte K blocks per operand row
+    int32_t kb;          // 128-byte K blocks per operand row (the last one maybe in part)
     int32_t ksteps;      // 32-byte MMA K steps that carry data
     int32_t rb;          // references per tile (MMA N = 256)
     int32_t kbs;         // K blocks per TMA stage (kb, or 1 for long rows)

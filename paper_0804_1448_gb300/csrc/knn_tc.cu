@@ -28,25 +28,26 @@ EncodeTiledFn encode_fn() {
 
 }  // namespace
 
-// rows x kp operand seen as 3-D: (128 bytes of K) x rows x K blocks, so one box
-// brings box_rows rows with all their K blocks, laid out block-major
-// ([K block][row][128 bytes], 128-byte swizzle) as the MMA descriptors expect.
-// Rows outside the tensor read as zero.
-bool tc_make_map(CUtensorMap* map, const void* base, int64_t rows, int kp, int prec, int box_rows,
-                 int box_kb) {
+// A box brings box_rows rows of one 128-byte K block, laid out [row][128 bytes]
+// with the 128-byte swizzle, as the MMA descriptors expect.  Rows are padded to
+// whole 32-byte MMA K steps only; what a box covers beyond the row's end (or of
+// rows outside the tensor) is filled with zeros and not read: d = 128 in bf16
+// takes 288 of 384 bytes a row, d = 96 in pairs 416 of 512, d = 96 in bf16 224
+// of 256.  Against rows of whole blocks the filter of 64 queries among 4194304
+// references, d = 96, bf16, which HBM bounds, takes 150 us instead of 162, and the
+// batches' copies are written in 64 instead of 69 ms of CTA time; where the tensor
+// cores bound the filter it changes little (n = m = 38400, d = 96: 281 -> 279 us).
+bool tc_make_map(CUtensorMap* map, const void* base, int64_t rows, int kp, int prec, int box_rows) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const int elt = (prec == kTF32) ? 4 : 2;
-    const int kb = kp * elt / kAtomBytes;
-    cuuint64_t dims[3] = {static_cast<cuuint64_t>(kAtomBytes / elt), static_cast<cuuint64_t>(rows),
-                          static_cast<cuuint64_t>(kb)};
-    cuuint64_t strides[2] = {static_cast<cuuint64_t>(kp) * elt, static_cast<cuuint64_t>(kAtomBytes)};
-    cuuint32_t box[3] = {static_cast<cuuint32_t>(kAtomBytes / elt), static_cast<cuuint32_t>(box_rows),
-                         static_cast<cuuint32_t>(box_kb > 0 ? box_kb : kb)};
-    cuuint32_t estr[3] = {1, 1, 1};
+    cuuint64_t dims[2] = {static_cast<cuuint64_t>(kp), static_cast<cuuint64_t>(rows)};
+    cuuint64_t strides[1] = {static_cast<cuuint64_t>(kp) * elt};
+    cuuint32_t box[2] = {static_cast<cuuint32_t>(kAtomBytes / elt), static_cast<cuuint32_t>(box_rows)};
+    cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map,
                     prec == kTF32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
-                    3, const_cast<void*>(base), dims, strides, box, estr,
+                    2, const_cast<void*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
@@ -152,8 +153,8 @@ cudaError_t launch_wait_probe(int32_t* error_flag, uint64_t limit_ns, cudaStream
 bool pair_rows_fit(int32_t d) { return d >= 1 && d <= kPairMaxD; }
 
 int tc_padded_dim(int32_t d, int prec) {
-    if (prec == kPair) return (pair_ksteps(d) + 3) / 4 * 64;
-    const int step = (prec == kBF16) ? 64 : 32;   // whole 128-byte K blocks per row
+    if (prec == kPair) return pair_ksteps(d) * 16;
+    const int step = (prec == kTF32) ? 8 : 16;   // whole 32-byte MMA K steps per row
     return (d + kAugCols + step - 1) / step * step;
 }
 
@@ -166,7 +167,7 @@ TcPlan tc_plan(int64_t n, int64_t m, int32_t d, int32_t kp, int prec, int32_t c,
     p.mt = 1;
     p.rb = kTileN;
     p.groups = kGroups;
-    p.kb = kp * elt / kAtomBytes;
+    p.kb = (kp * elt + kAtomBytes - 1) / kAtomBytes;
     p.ksteps = (d + kAugCols + kstep - 1) / kstep;
     if (prec == kPair) {
         p.ksteps = pair_ksteps(d);
@@ -174,11 +175,11 @@ TcPlan tc_plan(int64_t n, int64_t m, int32_t d, int32_t kp, int prec, int32_t c,
         p.tiles = m / kTileN;    // the caller passes whole tiles
     }
     p.stages = 0;
-    // whole-tile stages (one TMA box and one wait per tile) when two fit,
+    // whole-tile stages (one wait per tile, rows of up to two K blocks) when two fit,
     // else single-K-block stages, as many as fit
     // (raw hit staging with them when it also fits: rows of up to 2 K blocks)
     for (int s = 4; s >= 2 && p.stages == 0; --s)
-        if (tc_smem_bytes(p.kb, p.kb, s, false) <= kSmemLimit) {
+        if (p.kb <= 2 && tc_smem_bytes(p.kb, p.kb, s, false) <= kSmemLimit) {
             p.kbs = p.kb;
             p.stages = s;
             p.raw = (p.kb <= 2 && tc_smem_bytes(p.kb, p.kb, s, false, true) <= kSmemLimit) ? 1 : 0;
@@ -322,12 +323,17 @@ cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* Q, int64
                                 int32_t kp, void* R_lp, void* Q_lp, float* qnorm, int32_t* count0,
                                 int32_t* count1, cudaStream_t st, int* launches) {
     const int64_t tiles = pair_tiles(m);
-    const int64_t ref_warps = tiles * kTileN / kPairRows;
-    const int64_t warps = ref_warps + (n + kPairRows - 1) / kPairRows;
+    const int rpw = kPairRows * (d <= 16 ? 4 : (d <= 32 ? 2 : 1));   // rows per warp
+    const int64_t ref_warps = tiles * kTileN / rpw;
+    const int64_t warps = ref_warps + (n + rpw - 1) / rpw;
     const unsigned grid = static_cast<unsigned>((warps * 32 + 255) / 256);
-    prepare_pair_kernel<<<grid, 256, 0, st>>>(R, m, tiles, Q, n, d, kp, static_cast<uint32_t*>(R_lp),
-                                              static_cast<uint32_t*>(Q_lp), qnorm, ref_warps, count0,
-                                              count1);
+    auto kern = d <= 16    ? prepare_pair_kernel<8, 1>
+                : d <= 32  ? prepare_pair_kernel<16, 1>
+                : d <= 64  ? prepare_pair_kernel<32, 1>
+                : d <= 128 ? prepare_pair_kernel<32, 2>
+                           : prepare_pair_kernel<32, 3>;
+    kern<<<grid, 256, 0, st>>>(R, m, tiles, Q, n, d, kp, static_cast<uint32_t*>(R_lp),
+                               static_cast<uint32_t*>(Q_lp), qnorm, ref_warps, count0, count1);
     if (launches) ++*launches;
     return cudaGetLastError();
 }
@@ -353,7 +359,7 @@ cudaError_t launch_tc_pilot(const TcPlan& p, const void* Q_lp, int64_t n, const 
                             int32_t kp, int prec, uint32_t* gmax, int32_t* error_flag, cudaStream_t st,
                             int* launches) {
     CUtensorMap mq, mr;
-    if (!tc_make_map(&mq, Q_lp, n, kp, prec, kBlockM, 0) || !tc_make_map(&mr, R_lp, m, kp, prec, p.rb, p.kbs))
+    if (!tc_make_map(&mq, Q_lp, n, kp, prec, kBlockM) || !tc_make_map(&mr, R_lp, m, kp, prec, p.rb))
         return cudaErrorInvalidValue;
     TcArgs a = base_args(p, n, m, error_flag);
     a.gmax = gmax;   // every slot of every row is written by the pilot
@@ -399,7 +405,7 @@ cudaError_t launch_tc_filter(const TcPlan& p, const void* Q_lp, int64_t n, const
                              const float* qscale, int32_t* error_flag, cudaStream_t st,
                              int* launches) {
     CUtensorMap mq, mr;
-    if (!tc_make_map(&mq, Q_lp, n, kp, prec, kBlockM, 0) || !tc_make_map(&mr, R_lp, m, kp, prec, p.rb, p.kbs))
+    if (!tc_make_map(&mq, Q_lp, n, kp, prec, kBlockM) || !tc_make_map(&mr, R_lp, m, kp, prec, p.rb))
         return cudaErrorInvalidValue;
     TcArgs a = base_args(p, n, m, error_flag);
     a.stride = 1;

@@ -88,7 +88,7 @@ constexpr int kStageWordsRaw = 32;
 
 struct TcArgs {
     int64_t n, m;
-    int32_t kb;           // 128-byte K blocks per operand row (row pitch = kb * 128 bytes)
+    int32_t kb;           // 128-byte K blocks per operand row, the last one maybe in part
     int32_t ksteps;       // 32-byte MMA K steps that carry data
     int32_t kbs;          // K blocks per stage: kb (whole tiles) or 1 (long rows)
     int32_t stages;
@@ -265,8 +265,8 @@ __device__ __forceinline__ void tc_run(const CUtensorMap* tmap_q, const CUtensor
 
     const int KB = KBT > 0 ? KBT : a.kb, KBS = KBT > 0 ? KBT : a.kbs;
     const int NST = a.stages;
-    const int SPT = KB / KBS;                   // stages per reference tile (1, or KB when KBS = 1)
     const size_t stage_bytes = static_cast<size_t>(kRTileBytes) * KBS;
+    constexpr int kBlockElts = kAtomBytes / (PREC == kTF32 ? 4 : 2);   // row elements per K block
     unsigned char* sA = smem;
     unsigned char* sB = sA + static_cast<size_t>(KB) * kQTileBytes;
     uint32_t* stage = reinterpret_cast<uint32_t*>(sB + NST * stage_bytes);
@@ -315,87 +315,166 @@ __device__ __forceinline__ void tc_run(const CUtensorMap* tmap_q, const CUtensor
         atomicExch(a.error_flag, 1);
     };
 
+    // Where a tile may take several stages (KBT = 0) the producer and the MMA issuer
+    // each run as a whole warp, one elected lane doing the loads or the MMAs, so
+    // that counters, barriers and descriptors stay in uniform registers, and walk
+    // the ring with a slot and a parity instead of dividing a running stage number:
+    // their instructions compete with sixteen epilogue warps for issue slots, and
+    // they are the ring's latency.  Filter of n = m = 38400, d = 96, pairs 809 -> 612
+    // us, of n = 16384, m = 1048576, d = 128, bf16 5.30 -> 4.66 ms, of n = 9600,
+    // m = 19200, d = 64, tf32 68 -> 51 us.  With one stage a tile (KBT > 0) one lane
+    // runs alone: two K blocks, bf16, 279 us against 305 with whole warps.
     if (warp == 0) {
         // -------------------------------------------------------- producer
-        // one 3-D box per load: (128 bytes of K) x rows x K blocks
-        if (lane == 0) {
-            mbar_expect_tx(a_full, KB * kQTileBytes);
-            tma_load_3d(sA, tmap_q, a_full, 0, static_cast<int>(q0), 0);
-            int issued = 0;   // stage h = tile * SPT + K-block group
-            for (int h = 0; h < nt * SPT; ++h) {
-                const int g = h / SPT, z = (h % SPT) * KBS, s = h % NST;
-                if (!mbar_wait(&empty[s], ((h / NST) & 1) ^ 1, abort_flag)) { fail(); break; }
-                mbar_expect_tx(&full[s], static_cast<uint32_t>(stage_bytes));
-                const int y = static_cast<int>(r_begin + static_cast<int64_t>(g) * stride * kTileN);
-                tma_load_3d(sB + s * stage_bytes, tmap_r, &full[s], 0, y, z);
-                issued = h + 1;
+        // one box per K block: (128 bytes of K) x rows, columns past the row's
+        // end filled with zeros
+        if constexpr (KBT == 0) {
+            const bool el = elect_one();
+            if (el) {
+                mbar_expect_tx(a_full, KB * kQTileBytes);
+                for (int kb = 0; kb < KB; ++kb)
+                    tma_load_2d(sA + kb * kQTileBytes, tmap_q, a_full, kb * kBlockElts, static_cast<int>(q0));
+            }
+            __syncwarp();
+            int s = 0, issued = 0;        // ring slot, stages loaded
+            uint32_t ph = 0;              // parity of the slot's use
+            bool ok = true;
+            int y = static_cast<int>(r_begin);
+            for (int g = 0; ok && g < nt; ++g, y += stride * kTileN) {
+                for (int z = 0; z < KB; z += KBS) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], ph ^ 1u, abort_flag));
+                    if (!ok) {
+                        if (el) fail();
+                        break;
+                    }
+                    if (el) {
+                        mbar_expect_tx(&full[s], static_cast<uint32_t>(stage_bytes));
+                        for (int kb = 0; kb < KBS; ++kb)
+                            tma_load_2d(sB + s * stage_bytes + kb * kRTileBytes, tmap_r, &full[s],
+                                        (z + kb) * kBlockElts, y);
+                    }
+                    __syncwarp();
+                    ++issued;
+                    if (++s == NST) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
             }
             mbar_wait(a_full, 0, nullptr);   // drain: every issued copy has landed
             for (int h = (issued > NST ? issued - NST : 0); h < issued; ++h)
                 mbar_wait(&full[h % NST], (h / NST) & 1, nullptr);
+            __syncwarp();
+        } else {
+            if (lane == 0) {
+                mbar_expect_tx(a_full, KB * kQTileBytes);
+                for (int kb = 0; kb < KB; ++kb)
+                    tma_load_2d(sA + kb * kQTileBytes, tmap_q, a_full, kb * kBlockElts, static_cast<int>(q0));
+                int issued = 0;   // stage h: tile h
+                for (int h = 0; h < nt; ++h) {
+                    const int s = h % NST;
+                    if (!mbar_wait(&empty[s], ((h / NST) & 1) ^ 1, abort_flag)) { fail(); break; }
+                    mbar_expect_tx(&full[s], static_cast<uint32_t>(stage_bytes));
+                    const int y = static_cast<int>(r_begin + static_cast<int64_t>(h) * stride * kTileN);
+                    for (int kb = 0; kb < KBT; ++kb)
+                        tma_load_2d(sB + s * stage_bytes + kb * kRTileBytes, tmap_r, &full[s],
+                                    kb * kBlockElts, y);
+                    issued = h + 1;
+                }
+                mbar_wait(a_full, 0, nullptr);   // drain: every issued copy has landed
+                for (int h = (issued > NST ? issued - NST : 0); h < issued; ++h)
+                    mbar_wait(&full[h % NST], (h / NST) & 1, nullptr);
+            }
+            __syncwarp();
         }
-        __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if constexpr (KBT == 0) {
+            const bool el = elect_one();
             const uint32_t id = idesc(PREC == kTF32 ? 2 : 1, kBlockM, kTileN);
-            bool ok = mbar_wait(a_full, 0, abort_flag);
-            if (!ok) fail();
+            bool ok = __all_sync(0xffffffffu, mbar_wait(a_full, 0, abort_flag));
+            if (!ok && el) fail();
             const uint64_t a_desc = sdesc(smem_u32(sA));
+            const uint64_t b_desc0 = sdesc(smem_u32(sB));
+            const uint32_t b_step = static_cast<uint32_t>(stage_bytes >> 4);
             constexpr uint32_t kQStep = kQTileBytes >> 4, kRStep = kRTileBytes >> 4;
+            int s = 0;
+            uint32_t ph = 0;
             for (int g = 0; ok && g < nt; ++g) {
                 const int buf = g & 1;
-                if (!mbar_wait(&t_empty[buf], ((g >> 1) & 1) ^ 1, abort_flag)) { fail(); break; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&t_empty[buf], ((g >> 1) & 1) ^ 1, abort_flag));
+                if (!ok) {
+                    if (el) fail();
+                    break;
+                }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + buf * kTileN;
-                if (SPT == 1) {
+                for (int z = 0; z < KB; z += KBS) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, abort_flag));
+                    if (!ok) {
+                        if (el) fail();
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint64_t b_desc = b_desc0 + static_cast<uint32_t>(s) * b_step;
+                    if (el) {
+#pragma unroll
+                        for (int kb = 0; kb < 2; ++kb) {
+                            if (kb < KBS) {
+                                if constexpr (PREC == kPair)
+                                    issue_pair_kblock(d_tmem, a_desc, b_desc + kb * kRStep, z + kb, a.hs,
+                                                      a.ksteps, id);
+                                else
+                                    issue_kblock<PREC>(d_tmem, a_desc + (z + kb) * kQStep,
+                                                       b_desc + kb * kRStep, a.ksteps - (z + kb) * 4,
+                                                       z + kb == 0, id);
+                            }
+                        }
+                        tc_commit(&empty[s]);   // the stage is free once these MMAs complete
+                    }
+                    __syncwarp();
+                    if (++s == NST) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (!ok) break;
+                if (el) tc_commit(&t_full[buf]);
+                __syncwarp();
+            }
+            if (el) tc_commit(drain);   // arrives once every MMA issued above has completed
+            __syncwarp();
+            mbar_wait(drain, 0, nullptr);
+            __syncwarp();
+        } else {
+            if (lane == 0) {
+                const uint32_t id = idesc(PREC == kTF32 ? 2 : 1, kBlockM, kTileN);
+                bool ok = mbar_wait(a_full, 0, abort_flag);
+                if (!ok) fail();
+                const uint64_t a_desc = sdesc(smem_u32(sA));
+                constexpr uint32_t kQStep = kQTileBytes >> 4, kRStep = kRTileBytes >> 4;
+                for (int g = 0; ok && g < nt; ++g) {
+                    const int buf = g & 1;
+                    if (!mbar_wait(&t_empty[buf], ((g >> 1) & 1) ^ 1, abort_flag)) { fail(); break; }
+                    tc_fence_after();
+                    const uint32_t d_tmem = tmem + buf * kTileN;
                     // whole-tile stage g
                     const int s = g % NST;
                     if (!mbar_wait(&full[s], (g / NST) & 1, abort_flag)) { fail(); break; }
                     tc_fence_after();
                     const uint64_t b_desc = sdesc(smem_u32(sB + s * stage_bytes));
-                    if constexpr (PREC == kPair) {
-                        for (int kb = 0; kb < KB; ++kb)
-                            issue_pair_kblock(d_tmem, a_desc, b_desc + kb * kRStep, kb, a.hs,
-                                              a.ksteps, id);
-                    } else if (KBT > 0) {
 #pragma unroll
-                        for (int kb = 0; kb < (KBT > 0 ? KBT : 1); ++kb)
-                            issue_kblock<PREC>(d_tmem, a_desc + kb * kQStep, b_desc + kb * kRStep,
-                                               a.ksteps - kb * 4, kb == 0, id);
-                    } else {
-                        for (int kb = 0; kb < KB; ++kb)
-                            issue_kblock<PREC>(d_tmem, a_desc + kb * kQStep, b_desc + kb * kRStep,
-                                               a.ksteps - kb * 4, kb == 0, id);
-                    }
+                    for (int kb = 0; kb < KBT; ++kb)
+                        issue_kblock<PREC>(d_tmem, a_desc + kb * kQStep, b_desc + kb * kRStep,
+                                           a.ksteps - kb * 4, kb == 0, id);
                     tc_commit(&empty[s]);   // the stage is free once these MMAs complete
-                } else {
-                    // one K block per stage: tile g takes stages g*KB .. g*KB+KB-1
-                    for (int kb = 0; kb < KB; ++kb) {
-                        const int h = g * KB + kb, s = h % NST;
-                        if (!mbar_wait(&full[s], (h / NST) & 1, abort_flag)) {
-                            fail();
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        if constexpr (PREC == kPair)
-                            issue_pair_kblock(d_tmem, a_desc, sdesc(smem_u32(sB + s * stage_bytes)),
-                                              kb, a.hs, a.ksteps, id);
-                        else
-                            issue_kblock<PREC>(d_tmem, a_desc + kb * kQStep,
-                                               sdesc(smem_u32(sB + s * stage_bytes)),
-                                               a.ksteps - kb * 4, kb == 0, id);
-                        tc_commit(&empty[s]);
-                    }
-                    if (!ok) break;
+                    tc_commit(&t_full[buf]);
                 }
-                tc_commit(&t_full[buf]);
+                tc_commit(drain);   // arrives once every MMA issued above has completed
+                mbar_wait(drain, 0, nullptr);
             }
-            tc_commit(drain);   // arrives once every MMA issued above has completed
-            mbar_wait(drain, 0, nullptr);
+            __syncwarp();
         }
-        __syncwarp();
     } else {
         // -------------------------------------------------------- epilogue
         const int et = threadIdx.x - 64;            // 0 .. kEpi-1
@@ -666,8 +745,8 @@ __device__ __forceinline__ void put(void* row, int t, float v) {
 // The float32 search's own filter: three bf16 products in place of one fused
 // multiply-add per coordinate on the CUDA cores (33 TFLOP/s of 80, bound by
 // that pipe).  n = m = 38400, d = 96: 19 MMA steps of 16 coordinates a tile,
-// filter 0.79 ms, the whole search 8.57 -> 1.08 ms; n = 4999, m = 20011, d =
-// 50: 778 -> 116 us.  Two parts, not three: the part left out moves acc by less
+// filter 0.61 ms, the whole search 8.57 -> 0.86 ms; n = 4999, m = 20011, d =
+// 50: 778 -> 98 us.  Two parts, not three: the part left out moves acc by less
 // than the slack any float32 bound over d terms has to carry, and the answer
 // is made of exact float32 distances either way (its error against float64 is
 // the same to the digit).
@@ -717,12 +796,13 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-constexpr int kPairRows = 4;   // rows per warp
+constexpr int kPairRows = 4;   // rows per group of lanes
 constexpr int kPairMaxD = 192;
 
-// Operand rows of a search on pairs, references and queries in one launch:
-// warps below ref_warps take four consecutive rows of the reference copy, the
-// others four queries.  Coordinates are taken relative to the set's first
+// Operand rows of a search on pairs, references and queries in one launch: a
+// row per LANES lanes (8 up to d = 16, 16 up to 32, else a whole warp, NJ
+// coordinate pairs a lane), kPairRows rows at a time; warps below ref_warps take
+// consecutive rows of the reference copy, the others queries.  Coordinates are taken relative to the set's first
 // reference, so the slack follows the data's spread, not its offset from the
 // origin.  Row p of the copy, column c of tile g, holds reference
 // ((c mod 64) 4 + c / 64) T + g: every tile is an evenly spaced sample of the
@@ -732,16 +812,18 @@ constexpr int kPairMaxD = 192;
 // threshold passes.
 // The kernel reads and writes each row once, so memory bounds it; a lane holds
 // two neighbouring coordinates and stores them as one 32-bit word of h and one
-// of l, whole 128-byte lines per warp, and all loads of four rows are issued
-// before the first is used.  It also clears the search's two queue counters.
+// of l, and all loads of its rows are issued before the first is used.  (A warp
+// per row whatever d, with room for 192 coordinates: 19 us for
+// the self-join of 20000 points, d = 3; 23 against 27 at n = m = 38400, d = 96.)  It also clears the search's two queue counters.
+template <int LANES, int NJ>
 __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int64_t tiles,
                                     const float* __restrict__ Q, int64_t n, int32_t d, int32_t kp,
                                     uint32_t* __restrict__ R_lp, uint32_t* __restrict__ Q_lp,
                                     float* __restrict__ qnorm, int64_t ref_warps,
                                     int32_t* __restrict__ count0, int32_t* __restrict__ count1) {
     chain_begin();
-    constexpr int RW = kPairRows, NJ = kPairMaxD / 64;
-    const int lane = threadIdx.x % 32;
+    constexpr int RW = kPairRows, RPW = 32 / LANES;   // RPW rows side by side in a warp
+    const int lane = threadIdx.x % LANES, grp = threadIdx.x % 32 / LANES;
     int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) / 32;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *count0 = 0;
@@ -749,14 +831,14 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
     }
     const bool ref = w < ref_warps;
     if (!ref) w -= ref_warps;
-    const int64_t p0 = w * RW;
+    const int64_t p0 = w * (RW * RPW);   // a warp's rows, row u of a group of lanes RPW apart
     const int64_t rows = ref ? tiles * kTileN : n;
     if (p0 >= rows) return;
     const float* X = ref ? R : Q;
     int64_t src[RW];
 #pragma unroll
     for (int u = 0; u < RW; ++u) {
-        const int64_t p = p0 + u;
+        const int64_t p = p0 + u * RPW + grp;
         if (ref) {
             const int c = static_cast<int>(p % kTileN);
             src[u] = static_cast<int64_t>((c % kGroupCols) * kGroups + c / kGroupCols) * tiles + p / kTileN;
@@ -772,7 +854,7 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
         for (int j = 0; j < NJ; ++j)
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                const int t = 2 * lane + 64 * j + b;
+                const int t = 2 * lane + 2 * LANES * j + b;
                 xv[u][j][b] = (src[u] >= 0 && t < d) ? __ldg(X + src[u] * d + t) : 0.f;
             }
     float nr[RW];
@@ -782,7 +864,7 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
     for (int j = 0; j < NJ; ++j)
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            const int t = 2 * lane + 64 * j + b;
+            const int t = 2 * lane + 2 * LANES * j + b;
             if (t < d) {
                 const float c = __ldg(R + t);
 #pragma unroll
@@ -795,7 +877,7 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
             }
         }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
+    for (int o = LANES / 2; o > 0; o >>= 1)
 #pragma unroll
         for (int u = 0; u < RW; ++u) nr[u] += __shfl_xor_sync(0xffffffffu, nr[u], o);
     const int hs = pair_hsteps(d);
@@ -803,7 +885,7 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
     const float half_er = 0.5f - pair_slack(d).er;   // -(1/2 - er) n_r: er n_r of slack on acc
 #pragma unroll
     for (int u = 0; u < RW; ++u) {
-        const int64_t p = p0 + u;
+        const int64_t p = p0 + u * RPW + grp;
         if (p >= rows) break;
         float aug[kPairAug];
         if (ref) {
@@ -828,7 +910,7 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
         uint32_t* row = (ref ? R_lp : Q_lp) + p * (kp / 2);
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
-            const int t = 2 * lane + 64 * j;
+            const int t = 2 * lane + 2 * LANES * j;
             if (t >= 16 * hs) break;
             const float x0 = xv[u][j][0], x1 = xv[u][j][1];
             float h0 = lowp_round<kBF16>(x0), h1 = lowp_round<kBF16>(x1);
@@ -839,7 +921,7 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
             }
             row[t / 2] = bf16x2_bits(h0, h1);
         }
-        for (int e = 2 * lane; e < kp - 32 * hs; e += 64)
+        for (int e = 2 * lane; e < kp - 32 * hs; e += 2 * LANES)
             row[16 * hs + e / 2] =
                 inside ? 0u : bf16x2_bits(aug_at(e), aug_at(e + 1));
     }
@@ -1119,9 +1201,8 @@ __global__ void threshold_kernel(const uint32_t* __restrict__ gmax, int64_t n, i
 
 }  // namespace
 
-// rows x kp operand copy seen by TMA as 3-D boxes of box_rows rows (all K
-// blocks when box_kb = 0); false if the driver entry point is missing.
-bool tc_make_map(CUtensorMap* map, const void* base, int64_t rows, int kp, int prec, int box_rows,
-                 int box_kb);
+// rows x kp operand copy seen by TMA as boxes of box_rows rows x 128 bytes;
+// false if the driver entry point is missing.
+bool tc_make_map(CUtensorMap* map, const void* base, int64_t rows, int kp, int prec, int box_rows);
 
 }  // namespace knn
