@@ -9,7 +9,7 @@ does not state its distribution).  One step is one complete search of all
 re-check and the output.  Inputs are resident in HBM when a step starts; L2 is
 flushed (256 MiB write) before every step, outside the timed window.
 
-Also reported: the float32 CUDA-core form on the same workload, the same
+Also reported: the float32 form on the same workload, the same
 search end to end through the C ABI with pinned host buffers (host<->device
 copies timed), the roofline fraction of the dominant kernel, and the oracle
 timed on the host cores on a bounded sample.
@@ -393,7 +393,7 @@ TABLE1_BF_CUDA = {
 
 def configs(args):
     """Timings of the forms and shapes beside the bench line, one JSON line:
-    config 1 (n = m = 1200, d = 8, k = 20: float32 CUDA-core and bf16 forms,
+    config 1 (n = m = 1200, d = 8, k = 20: float32 and bf16 forms,
     and the oracle on the host cores over all 1200 queries, on all cores and
     on one), config 2
     (n = m = 38400, d = 96, k = 20: float32 Euclidean, Manhattan and
@@ -769,7 +769,7 @@ def main():
                    else "bf16_tflops x 1.1/2.25 (nominal tf32:bf16 ratio)"),
                 "kernel_ms": filt_avg, "flops_per_launch": flops}
 
-    # ---- float32 CUDA-core form, same workload (the comparator)
+    # ---- float32 form, same workload (the comparator)
     ix32 = knn.Index(local, "fp32")
     ix32.set_reference(Rd)
     for _ in range(3):
