@@ -51,21 +51,26 @@ cudaError_t allow_smem(size_t smem) {
     return err;
 }
 
-// The kernels of one search run one after another on one stream, each launched
+// The kernels of one search run one after another on one stream, each set up
 // while its predecessor still runs (programmatic dependent launch): a kernel
-// calls chain_begin() before it touches memory, which lets its successor be
-// launched and waits until everything before it on the stream is done.  Every
-// kernel that launch_chained launches calls it, on every path that reads or
-// writes memory; the first kernel of a search is launched plainly, so a search
-// waits for whatever the caller's stream holds.  Searches with device buffers
-// are chained: n = m = 1200, d = 8 (three kernels) 32.5 -> 24.9 us, one query
-// among 5000 references, d = 8 (eight) 47 -> 33, n = 4999, m = 20011, d = 50 116
-// -> 99.  Those with host buffers are not (chain = false): their parts share the
-// SMs from two streams, and CTAs of one part's waiting kernels kept the other's
-// out (n = m = 38400, d = 96: 635 -> 660 us).
+// calls chain_begin() before it touches memory, which waits until everything
+// before it on the stream is done.  Every kernel that launch_chained launches
+// calls it, on every path that reads or writes memory; the first kernel of a
+// search is launched plainly, so a search waits for whatever the caller's stream
+// holds.  Searches with device buffers are chained: n = m = 1200, d = 8 (three
+// kernels) 32.5 -> 22.6 us, n = 4999, m = 20011, d = 50 116 -> 92.  Those with
+// host buffers are not (chain = false): the parts of a large one share the SMs
+// from two streams.
+// No kernel lets its successor in early (griddepcontrol.launch_dependents): its
+// CTAs would settle, waiting, on whatever SMs have room first, several on one,
+// and keep the other streams' kernels out.  With it the 4096 queries of m =
+// 20000, d = 96 that the exact fallback takes cost 73 ms instead of 38, n = 2000,
+// m = 9600, d = 64 in tf32 58 us instead of 48, and two handles searching at once
+// (n = 1024, m = 100000, d = 64, bf16) 69 us a search instead of 47; what it saves
+// is about 1 us a kernel where every grid is many waves long (n = m = 38400, d =
+// 96, bf16: 541 against 546 us).
 __device__ __forceinline__ void chain_begin() {
 #ifdef __CUDA_ARCH__
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 #endif
 }
