@@ -1009,7 +1009,7 @@ finalize_kernel(FinalizeArgs a, int P, int warps_per_block, int stage_entries) {
         const int count = *a.from.count;
         if (row >= count) return;
         q = a.from.list[row];
-        if (count <= kDirectQueue) {   // too few for the select: no candidates to finish
+        if (count <= a.direct) {   // too few for the select: no candidates to finish
             if (lane == 0) queue_fallback(a, q, 3);
             return;
         }

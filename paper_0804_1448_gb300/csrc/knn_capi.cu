@@ -326,6 +326,7 @@ struct SearchPlan {
     int64_t chunk = 0;
     TcPlan plan{};
     int64_t fb_grid = 1;
+    int32_t direct = 0;      // filtered(): queues up to this long skip the select
     size_t off_cand = 0, off_ql = 0, off_gmax = 0, off_lists = 0, off_counts = 0, off_qs = 0;
     size_t off_rl = 0, off_queue = 0;   // operand pairs: reference copy; queued queries and their count
     size_t off_list = 0, off_scr = 0, off_fbdone = 0, off_q = 0, off_dist = 0, off_idx = 0;
@@ -417,6 +418,15 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
     p.fb_grid = fb_cap_bytes / (8 * m);
     if (p.fb_grid > 64) p.fb_grid = 64;
     if (p.fb_grid < 1) p.fb_grid = 1;
+    // What a filter leaves over: queues no longer than the fallback can spread
+    // over the GPU go straight to it where that is faster than the select.  The
+    // fallback ends with one CTA going over a query's m keys five times, 0.78 ns a
+    // reference (m = 1 million: 0.78 ms); the select's CTAs stream their split at
+    // 65 ns a reference or more and its finalize takes 0.2 ms: 0.45 ms for 16
+    // queries of m = 1 million, d = 2, k = 10 (227 splits), 4.9 ms at d = 128, k =
+    // 100 (32 splits), 0.3 ms at m = 100000, d = 8.
+    if (p.filtered() && m < (1 << 18) + 80 * p.chunk)
+        p.direct = std::min<int32_t>(kDirectMost, fallback_spread(static_cast<int32_t>(p.fb_grid)));
 
     // workspace layout
     Carve cv;
@@ -647,11 +657,12 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
         cs.chunk = sp.chunk;
         cs.exact = 1;
         cs.chain = chain ? 1 : 0;
-        KNN_CUDA(h, launch_cc_select(Qd, n, rv.R, m, d, metric, cs, st, l, queue));
+        KNN_CUDA(h, launch_cc_select(Qd, n, rv.R, m, d, metric, cs, st, l, queue, sp.direct));
         fa.use_hits = 0;
         fa.hits = HitLists{};
         fa.cand = cs;
         fa.from = queue;
+        fa.direct = sp.direct;
         KNN_CUDA(h, launch_finalize(fa, st, l));
         mark("cc_queued");
     } else {

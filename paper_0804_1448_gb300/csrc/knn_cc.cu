@@ -151,16 +151,16 @@ __device__ __forceinline__ float pair_hi(uint64_t v) { return __uint_as_float(st
 // threads below kTM (below ROWS, in a CTA's first tile) also sum the squares
 // of reference (query) tid's staged coordinates, its squared norm.
 // QUEUED: the CTA's queries are those of a queue (nothing to do while it is no
-// longer than kDirectQueue), candidate row i being that of the queue's i-th.
+// longer than direct), candidate row i being that of the queue's i-th.
 template <int METRIC, int ROWS, bool QUEUED>
 __global__ void __launch_bounds__(kThreads, CCShape<ROWS>::MINB)
 cc_select_kernel(const float* __restrict__ Q, int64_t n, const float* __restrict__ R,
-                 int64_t m, int32_t d, CandidateSet cand, QueryQueue from) {
+                 int64_t m, int32_t d, CandidateSet cand, QueryQueue from, int32_t direct) {
     chain_begin();
     if (cand.clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *cand.clear = 0;
     if constexpr (QUEUED) {
         const int count = *from.count;
-        if (count <= kDirectQueue || static_cast<int64_t>(blockIdx.x) * ROWS >= count) return;
+        if (count <= direct || static_cast<int64_t>(blockIdx.x) * ROWS >= count) return;
         n = count;
     }
     using S = CCShape<ROWS>;
@@ -438,24 +438,27 @@ cc_select_kernel(const float* __restrict__ Q, int64_t n, const float* __restrict
 template <int METRIC, int ROWS, bool QUEUED = false>
 cudaError_t launch_rows(const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
                         const CandidateSet& cand, cudaStream_t st,
-                        const QueryQueue& from = QueryQueue{}) {
+                        const QueryQueue& from = QueryQueue{}, int32_t direct = 0) {
     auto kern = cc_select_kernel<METRIC, ROWS, QUEUED>;
     const size_t smem = cc_smem_bytes<ROWS>(cand.c);
     cudaError_t err = allow_smem<cc_select_kernel<METRIC, ROWS, QUEUED>>(smem);
     if (err != cudaSuccess) return err;
     dim3 grid(static_cast<unsigned>((n + ROWS - 1) / ROWS), static_cast<unsigned>(cand.S));
-    if (QUEUED) return launch_chained(cand.chain != 0, kern, grid, dim3(kThreads), smem, st, Q, n, R, m, d, cand, from);
-    kern<<<grid, kThreads, smem, st>>>(Q, n, R, m, d, cand, from);   // a search's first kernel
+    if (QUEUED)
+        return launch_chained(cand.chain != 0, kern, grid, dim3(kThreads), smem, st, Q, n, R, m, d, cand,
+                              from, direct);
+    kern<<<grid, kThreads, smem, st>>>(Q, n, R, m, d, cand, from, 0);   // a search's first kernel
     return cudaGetLastError();
 }
 
 template <int METRIC>
 cudaError_t launch_metric(int rows, const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
-                          const CandidateSet& cand, cudaStream_t st, const QueryQueue& from) {
+                          const CandidateSet& cand, cudaStream_t st, const QueryQueue& from,
+                          int32_t direct) {
     if (from.list)
-        return rows == 128 ? launch_rows<METRIC, 128, true>(Q, n, R, m, d, cand, st, from)
-               : rows == 64 ? launch_rows<METRIC, 64, true>(Q, n, R, m, d, cand, st, from)
-                            : launch_rows<METRIC, 16, true>(Q, n, R, m, d, cand, st, from);
+        return rows == 128 ? launch_rows<METRIC, 128, true>(Q, n, R, m, d, cand, st, from, direct)
+               : rows == 64 ? launch_rows<METRIC, 64, true>(Q, n, R, m, d, cand, st, from, direct)
+                            : launch_rows<METRIC, 16, true>(Q, n, R, m, d, cand, st, from, direct);
     return rows == 128 ? launch_rows<METRIC, 128>(Q, n, R, m, d, cand, st)
            : rows == 64 ? launch_rows<METRIC, 64>(Q, n, R, m, d, cand, st)
                         : launch_rows<METRIC, 16>(Q, n, R, m, d, cand, st);
@@ -538,14 +541,14 @@ int cc_max_candidates() {
 
 cudaError_t launch_cc_select(const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
                              int32_t metric, const CandidateSet& cand, cudaStream_t st,
-                             int* launches, const QueryQueue& from) {
+                             int* launches, const QueryQueue& from, int32_t direct) {
     int64_t per_sm = 1;
     const int rows = cc_rows(n, cand.c, &per_sm);
     if (rows == 16 && cc_smem_bytes<16>(cand.c) > kSmemCap) return cudaErrorInvalidValue;
     if (launches) ++*launches;
-    if (metric == kL2) return launch_metric<kL2>(rows, Q, n, R, m, d, cand, st, from);
-    if (metric == kL1) return launch_metric<kL1>(rows, Q, n, R, m, d, cand, st, from);
-    return launch_metric<kLinf>(rows, Q, n, R, m, d, cand, st, from);
+    if (metric == kL2) return launch_metric<kL2>(rows, Q, n, R, m, d, cand, st, from, direct);
+    if (metric == kL1) return launch_metric<kL1>(rows, Q, n, R, m, d, cand, st, from, direct);
+    return launch_metric<kLinf>(rows, Q, n, R, m, d, cand, st, from, direct);
 }
 
 }  // namespace knn

@@ -127,7 +127,7 @@ cudaError_t launch_fallback_m(const FinalizeArgs& a, double* scratch, int32_t sl
     if (err != cudaSuccess) return err;
     // half of the scratch slots for spread queries, half for the rest (a lone
     // slot serves every queued query with one CTA)
-    const int32_t spread = slots >= 2 ? slots / 2 : 0;
+    const int32_t spread = fallback_spread(slots);
     const unsigned chunks = spread > 0 ? static_cast<unsigned>((a.m + kFbChunk - 1) / kFbChunk) : 1u;
     return launch_chained(a.chain != 0, fallback_kernel<METRIC>, dim3(chunks, static_cast<unsigned>(slots)),
                           dim3(kFbThreads), smem, st, a, scratch, done, spread);

@@ -162,13 +162,17 @@ struct HitLists {
 };
 
 // The queries one pass left to the next: list[0 .. *count).  A pass over a
-// queue does nothing while it holds kDirectQueue queries or fewer: those go
-// straight to the exact fallback, which spreads each over the GPU.
+// queue does nothing while it holds `direct` queries or fewer (an argument of
+// each pass): those go straight to the exact fallback.
 struct QueryQueue {
     int32_t* list;    // null: the pass covers every query
     int32_t* count;
 };
-constexpr int kDirectQueue = 32;
+// How many queued queries the exact fallback spreads over the GPU, given its
+// scratch slots (the others take one CTA each); and the most that a queue may
+// send it at once.
+inline int32_t fallback_spread(int32_t slots) { return slots >= 2 ? slots / 2 : 0; }
+constexpr int kDirectMost = 32;
 
 struct FinalizeArgs {
     int32_t use_hits;       // 0: candidates come from `cand`; 1: from `hits`
@@ -187,6 +191,7 @@ struct FinalizeArgs {
                                // the queue's i-th; null: all n
     int32_t leave;             // 1: fallback_list is the next pass's queue, not the exact
                                // fallback's (its queries are not counted as such)
+    int32_t direct;            // `from`: queues up to this long are not finished here
     unsigned long long* recheck_counter;
     unsigned long long* fallback_total;
     unsigned long long* fallback_reason;   // [4]: short list, overflow, wide cut, uncertified
@@ -204,10 +209,11 @@ struct FinalizeArgs {
 
 // CUDA-core fused distance + top-c.  Writes cand (exact = 1).
 // from.list: only the queue's queries, candidate row i being that
-// of its i-th.
+// of its i-th, and none while there are no more than `direct`.
 cudaError_t launch_cc_select(const float* Q, int64_t n, const float* R, int64_t m, int32_t d,
                              int32_t metric, const CandidateSet& cand, cudaStream_t st,
-                             int* launches, const QueryQueue& from = QueryQueue{});
+                             int* launches, const QueryQueue& from = QueryQueue{},
+                             int32_t direct = 0);
 
 // Manhattan and Chebyshev searches with a pilot threshold and hit lists
 // (knn_diff.cu), one list per query and split.

@@ -1,0 +1,68 @@
+"""What a float32 filter cannot certify (needs a GB300): the length of the queue
+that skips the CUDA-core select, and the select over a queue at the edges of its
+CTA shapes.  The rule is tests/parity.py's."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0804_1448_gb300 import inputs
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def knn():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0804_1448_gb300 import knn as mod
+    return mod
+
+
+def ladders(m, n, n_ladder, d=16, rungs=100, step=5e-7, seed=5):
+    """Uniform points; around each of n_ladder of the queries `rungs` references
+    at squared distances 0.01 + i step: more of them within the operand pairs'
+    slack (some 7e-5 here) than the filter keeps.  The select keeps as many in
+    every one of its splits, over which they are spread."""
+    rng = np.random.default_rng(seed)
+    Q = inputs.uniform(n, d, seed=seed + 1)
+    R = inputs.uniform(m, d, seed=seed + 2)
+    at = rng.permutation(m)[:n_ladder * rungs].reshape(n_ladder, rungs)
+    who = rng.permutation(n)[:n_ladder]
+    s = np.sqrt(0.01 + step * np.arange(rungs))
+    for q, rows in zip(who, at):
+        u = rng.standard_normal((rungs, d))
+        u /= np.linalg.norm(u, axis=1, keepdims=True)
+        R[rows] = (Q[q].astype(np.float64) + s[:, None] * u).astype(np.float32)
+    return R, Q
+
+
+def check(knn, R, Q, k, rows=None):
+    import torch
+    ix = knn.Index(0, "fp32")
+    ix.set_reference(torch.from_numpy(R).cuda())
+    dist, idx = ix.search(torch.from_numpy(Q).cuda(), k)
+    ix.sync()
+    st = ix.stats()
+    ix.close()
+    dist, idx = dist.cpu().numpy(), idx.cpu().numpy()
+    if rows is not None:
+        dist, idx, Q = dist[rows], idx[rows], Q[rows]
+    o_dist, o_idx = oracle.knn(R, Q, parity.oracle_k(k, R.shape[0]), "l2")
+    parity.compare(dist, idx, o_dist, o_idx, k, R.shape[0])
+    return st
+
+
+@pytest.mark.parametrize("m,direct", [(20000, True), (600000, False)])
+def test_short_queues_of_a_large_set_take_the_select(knn, m, direct):
+    """16 queries that the filter cannot certify: among 20000 references the
+    exact fallback spreads them over the GPU; among 600000 it would spread 6 and
+    read the whole set through one CTA for each of the others, and the select,
+    which certifies them all, is the faster form."""
+    R, Q = ladders(m, 16, 16)
+    st = check(knn, R, Q, 10)
+    if direct:
+        assert st["fallback_queries"] > 8
+    else:
+        assert st["fallback_queries"] == 0
