@@ -163,6 +163,17 @@ knn_status knn_sync(knn_handle h);
 knn_status knn_selftest_bounded_wait(knn_handle h, int32_t limit_ms);
 
 /*
+ * Self-test of the tensor cores' sums, on which the certificates of float32
+ * Euclidean searches rest: A (128 x 64) and B (256 x 64), host pointers, are
+ * rounded to bf16, and the first `steps` (1..4) steps of 16 columns of A B^T are
+ * multiplied and added up by one tensor-core instruction each, into D (128 x 256,
+ * host).  A search allows every step an error of 17 * 2^-24 of the largest among
+ * its products, the sum before it and the sum after it.  Synchronous.
+ * Errors: KNN_ERR_INVALID, KNN_ERR_OOM, KNN_ERR_CUDA, KNN_ERR_TIMEOUT.
+ */
+knn_status knn_selftest_mma(knn_handle h, const float* A, const float* B, int32_t steps, float* D);
+
+/*
  * The plan a search would run with, without running it (host only; no GPU,
  * no handle): how knn_search of n queries against m references of dimension
  * d would be split and staged on a GPU with num_sms SMs, in the given

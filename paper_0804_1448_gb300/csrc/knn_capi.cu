@@ -1611,6 +1611,24 @@ knn_status knn_selftest_bounded_wait(knn_handle h, int32_t limit_ms) {
     return knn_sync(h);
 }
 
+knn_status knn_selftest_mma(knn_handle h, const float* A, const float* B, int32_t steps, float* D) {
+    if (!h || !A || !B || !D || steps < 1 || steps > 4) return KNN_ERR_INVALID;
+    KNN_CUDA(h, cudaSetDevice(h->device));
+    constexpr size_t na = 128 * 64, nb = 256 * 64, nd = 128 * 256;
+    float* buf = nullptr;
+    KNN_CUDA(h, cudaMalloc(&buf, (na + nb + nd) * sizeof(float)));
+    cudaError_t err = cudaMemcpyAsync(buf, A, na * sizeof(float), cudaMemcpyHostToDevice, h->stream);
+    if (err == cudaSuccess)
+        err = cudaMemcpyAsync(buf + na, B, nb * sizeof(float), cudaMemcpyHostToDevice, h->stream);
+    if (err == cudaSuccess)
+        err = launch_mma_probe(buf, buf + na, steps, buf + na + nb, &h->counters->error_flag, h->stream);
+    if (err == cudaSuccess)
+        err = cudaMemcpyAsync(D, buf + na + nb, nd * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
+    const knn_status s = err == cudaSuccess ? knn_sync(h) : cuda_fail(h, err, "tensor-core self-test");
+    cudaFree(buf);
+    return s;
+}
+
 knn_status knn_selftest_batch_queue(knn_handle h, int32_t limit_ms) {
     if (!h || limit_ms < 1 || limit_ms > 1000) return KNN_ERR_INVALID;
     KNN_CUDA(h, cudaSetDevice(h->device));

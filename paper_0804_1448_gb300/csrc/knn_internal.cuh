@@ -283,6 +283,10 @@ cudaError_t launch_whiten(const float* X, int64_t rows, int32_t d, const float* 
 // One bounded mbarrier wait that nothing completes: raises *error_flag after
 // limit_ns (the failure path of every device-side wait, exercised on purpose).
 cudaError_t launch_wait_probe(int32_t* error_flag, uint64_t limit_ns, cudaStream_t st);
+// One tile of bf16 MMA steps (knn_selftest_mma): D[128][256] = the first `steps`
+// (1 to 4) steps of 16 columns of A[128][64] times B[256][64], one after another.
+cudaError_t launch_mma_probe(const float* A, const float* B, int32_t steps, float* D,
+                             int32_t* error_flag, cudaStream_t st);
 
 // Self-join rows: the n x (k+1) result of searching R against itself, minus
 // each row's own index (or its last entry), into n x k outputs.

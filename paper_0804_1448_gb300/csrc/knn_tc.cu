@@ -150,6 +150,68 @@ cudaError_t launch_wait_probe(int32_t* error_flag, uint64_t limit_ns, cudaStream
     return cudaGetLastError();
 }
 
+// Self-test of the tensor cores' sums: the operands as the search kernels lay
+// them out (one K block, 128-byte swizzle), `steps` MMA steps of 16 products into
+// one accumulator, the accumulator as it stands.
+__global__ void __launch_bounds__(128)
+mma_probe_kernel(const float* __restrict__ A, const float* __restrict__ B, int32_t steps,
+                 float* __restrict__ D, int32_t* error_flag) {
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t slot;
+    const uint32_t raw = smem_u32(smem_raw);
+    unsigned char* sA = smem_raw + (((raw + 1023u) & ~1023u) - raw);
+    unsigned char* sB = sA + kQTileBytes;
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    for (int e = tid; e < (kBlockM + kTileN) * 64; e += 128) {
+        const bool a = e < kBlockM * 64;
+        const int i = a ? e : e - kBlockM * 64, r = i / 64, c = i % 64;
+        __nv_bfloat16* row = reinterpret_cast<__nv_bfloat16*>((a ? sA : sB) + r * kAtomBytes);
+        row[((c / 8) ^ (r & 7)) * 8 + c % 8] = __float2bfloat16_rn((a ? A : B)[i]);
+    }
+    if (tid == 0) {
+        mbar_init(&bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(&slot, kTileN);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = slot;
+    if (tid == 0) {
+        const uint64_t a_desc = sdesc(smem_u32(sA)), b_desc = sdesc(smem_u32(sB));
+        for (int s = 0; s < steps; ++s)
+            mma<kBF16>(tmem, a_desc + 2 * s, b_desc + 2 * s, idesc(1, kBlockM, kTileN), s == 0 ? 0u : 1u);
+        tc_commit(&bar);
+    }
+    __syncwarp();
+    if (!mbar_wait(&bar, 0, nullptr)) atomicExch(error_flag, 1);
+    __syncwarp();
+    tc_fence_after();
+    for (int c = 0; c < kTileN; c += 32) {
+        uint32_t r[32];
+        tmem_ld32u(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c, r);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) D[(warp * 32 + lane) * kTileN + c + i] = __uint_as_float(r[i]);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tmem, kTileN);
+    }
+}
+
+cudaError_t launch_mma_probe(const float* A, const float* B, int32_t steps, float* D,
+                             int32_t* error_flag, cudaStream_t st) {
+    constexpr size_t smem = kQTileBytes + kRTileBytes + 1024;
+    cudaError_t err = allow_smem<mma_probe_kernel>(smem);
+    if (err != cudaSuccess) return err;
+    mma_probe_kernel<<<1, 128, smem, st>>>(A, B, steps, D, error_flag);
+    return cudaGetLastError();
+}
+
 bool pair_rows_fit(int32_t d) { return d >= 1 && d <= kPairMaxD; }
 
 int tc_padded_dim(int32_t d, int prec) {

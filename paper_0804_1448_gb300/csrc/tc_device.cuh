@@ -773,18 +773,22 @@ __host__ __device__ constexpr int pair_ksteps(int d) {
 
 // Error bound of acc = q'.r' - n_r/2 + t as the tensor cores return it, as
 // eq n_q + er n_r + acc |t|.  Besides the words left out: each of the
-// 3 hs + 1 MMA steps adds 16 exact products to the accumulator, 17 addends each
-// cut at no less than 2^-23 of the largest partial sum, which is at most
-// 1.02 (n_q + n_r) / 2 + n_r / 2 + |t|; the norms are float32 sums of d squares
-// ((d + 8) 2^-24), cut to 24 bits; and taking q and r relative to a centre
-// rounds each coordinate once, 4 * 2^-24 (n_q + n_r) of the squared distance.
+// 3 hs MMA steps (and the one of the extra words, if any) adds 16 exact products
+// to the accumulator, with an error of at most 17 * 2^-24 of the largest among
+// the products and the sums before and after, which is at most 1.02 (n_q +
+// n_r) / 2 + n_r / 2 + |t|.  (Measured on GB300 with knn_selftest_mma: the 17
+// addends are cut at 2^-25 of the largest's power of two and their sum at 2^-23
+// of its own, 10.5 * 2^-24 together; the worst of the operands tried came to 0.43 of
+// the bound.)  The norms are float32 sums of d squares ((d + 8) 2^-24), cut to 24
+// bits; and taking q and r relative to a centre rounds each coordinate once, 4 *
+// 2^-24 (n_q + n_r) of the squared distance.
 struct PairSlack {
     float eq, er, acc;
 };
 __host__ __device__ inline PairSlack pair_slack(int d) {
     constexpr float u = 5.9604644775390625e-8f;   // 2^-24
     PairSlack s;
-    s.acc = 34.f * u * static_cast<float>(3 * pair_hsteps(d) + 1);
+    s.acc = 17.f * u * static_cast<float>(3 * pair_hsteps(d) + (pair_aug_inside(d) ? 0 : 1));
     const float common = 1.505f * 256.f * u + static_cast<float>(d + 16) * u;
     s.eq = common + 0.51f * s.acc;
     s.er = common + 1.02f * s.acc;

@@ -93,6 +93,7 @@ _SIGS = {
     "knn_sync": (ctypes.c_int, [_H]),
     "knn_selftest_bounded_wait": (ctypes.c_int, [_H, _i32]),
     "knn_selftest_batch_queue": (ctypes.c_int, [_H, _i32]),
+    "knn_selftest_mma": (ctypes.c_int, [_H, _P, _P, _i32, _P]),
     "knn_explain_plan": (ctypes.c_int, [_i64, _i64, _i32, _i32, ctypes.c_int, _i32, _i32, _i32,
                                         ctypes.POINTER(knn_plan)]),
     "knn_set_precision": (ctypes.c_int, [_H, _i32]),
@@ -129,6 +130,7 @@ knn_search = _lib.knn_search
 knn_sync = _lib.knn_sync
 knn_selftest_bounded_wait = _lib.knn_selftest_bounded_wait
 knn_selftest_batch_queue = _lib.knn_selftest_batch_queue
+knn_selftest_mma = _lib.knn_selftest_mma
 knn_explain_plan = _lib.knn_explain_plan
 
 knn_set_precision = _lib.knn_set_precision
