@@ -54,12 +54,14 @@ struct RefSet {
     int32_t kp = 0;               // padded row length of R_lp
     int lp_prec = 0;              // 0: none, kTF32, kBF16
     uint32_t* rmax2 = nullptr;    // device: largest ||r||^2 (float bits)
+    float* centre = nullptr;      // [d], of the operand pairs
     ~RefSet() {
         cudaSetDevice(device);
         if (R) cudaFree(R);
         if (r_norms) cudaFree(r_norms);
         if (R_lp) cudaFree(R_lp);
         if (rmax2) cudaFree(rmax2);
+        if (centre) cudaFree(centre);
     }
 };
 
@@ -223,8 +225,9 @@ knn_status build_lowp_on(knn_ctx* h, std::shared_ptr<RefSet>& ref, int prec) {
 
 knn_status build_lowp(knn_ctx* h, int prec) { return build_lowp_on(h, h->ref, prec); }
 
-// A reference set owning a float32 copy of R (m x d) and zeroed norm buffers;
-// src_kind is the cudaMemcpy kind of the copy.
+// A reference set owning a float32 copy of R (m x d), its centre and zeroed norm
+// buffers; src_kind is the cudaMemcpy kind of the copy.  Without R the caller
+// fills rs->R and then sets the centre (launch_centre).
 knn_status new_refset(knn_ctx* h, const float* R, int64_t m, int32_t d, cudaMemcpyKind src_kind,
                       std::shared_ptr<RefSet>* out) {
     auto rs = std::make_shared<RefSet>();
@@ -237,7 +240,13 @@ knn_status new_refset(knn_ctx* h, const float* R, int64_t m, int32_t d, cudaMemc
     KNN_CUDA(h, cudaMalloc(&rs->rmax2, sizeof(uint32_t)));
     KNN_CUDA(h, cudaMemsetAsync(rs->r_norms, 0, mpad * sizeof(float), h->stream));
     KNN_CUDA(h, cudaMemsetAsync(rs->rmax2, 0, sizeof(uint32_t), h->stream));
-    if (R) KNN_CUDA(h, cudaMemcpyAsync(rs->R, R, bytes, src_kind, h->stream));
+    KNN_CUDA(h, cudaMalloc(&rs->centre, static_cast<size_t>(d) * sizeof(float)));
+    if (R) {
+        KNN_CUDA(h, cudaMemcpyAsync(rs->R, R, bytes, src_kind, h->stream));
+        int l = 0;
+        KNN_CUDA(h, launch_centre(rs->R, m, d, rs->centre, h->stream, &l));
+        h->launches += l;
+    }
     KNN_CUDA(h, cudaStreamSynchronize(h->stream));
     rs->m = m;
     rs->d = d;
@@ -256,6 +265,7 @@ knn_status ensure_mref(knn_ctx* h) {
     if (s != KNN_OK) return s;
     int l = 0;
     KNN_CUDA(h, launch_whiten(h->ref->R, h->ref->m, h->ref->d, h->mahal_L, w->R, h->stream, &l));
+    KNN_CUDA(h, launch_centre(w->R, w->m, w->d, w->centre, h->stream, &l));
     KNN_CUDA(h, cudaStreamSynchronize(h->stream));
     h->launches += l;
     h->mref = std::move(w);
@@ -511,6 +521,7 @@ struct RefView {
     void* R_lp;
     int32_t kp;
     const uint32_t* rmax2;
+    const float* centre;   // operand pairs only
 };
 
 // Enqueue the kernels of one planned search on st: Q, dd, id on the device,
@@ -552,7 +563,7 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
         HitScale qs_prep = qs;   // the threshold pass sets B when there is one
         if (plan.pilot) qs_prep.qscale = nullptr;
         if (sp.pair)
-            KNN_CUDA(h, launch_prepare_pair(rv.R, m, Qd, n, d, kp, ws + sp.off_rl, Ql, qs.qscale,
+            KNN_CUDA(h, launch_prepare_pair(rv.R, m, rv.centre, Qd, n, d, kp, ws + sp.off_rl, Ql, qs.qscale,
                                             queue.count, fallback_count, st, l));
         else
             KNN_CUDA(h, launch_prepare_query(Qd, n, d, kp, prec, Ql, qs_prep, Q_copy, fallback_count,
@@ -771,7 +782,7 @@ knn_status enqueue_instance(knn_ctx* h, const knn_instance& x, const BatchPlan& 
     if (x.n == 0) return KNN_OK;
     const SearchPlan& sp = bp.sp[i];
     unsigned char* ws = h->ws;
-    RefView rv{x.R, x.m, x.d, nullptr, 0, nullptr};
+    RefView rv{x.R, x.m, x.d, nullptr, 0, nullptr, nullptr};
     if (sp.tensor) {
         rv.R_lp = ws + bp.lp[i];
         rv.kp = sp.kp;
@@ -1261,7 +1272,7 @@ knn_status knn_search(knn_handle h, const float* Q, int64_t n, int32_t d, int32_
         Qd = h->qw;
         stage(h, st, "whiten_q");
     }
-    RefView rv{rs.R, rs.m, rs.d, rs.R_lp, rs.kp, rs.rmax2};
+    RefView rv{rs.R, rs.m, rs.d, rs.R_lp, rs.kp, rs.rmax2, rs.centre};
     // Queries and outputs both in pinned host memory, read and written in
     // place: the link moves the queries at a fraction of the rate the kernels
     // use them, so a large search runs in parts (whole 128-query tiles), each
@@ -1539,7 +1550,7 @@ knn_status knn_search_self(knn_handle h, int32_t k, knn_metric metric, float* di
     int32_t* itmp = reinterpret_cast<int32_t*>(ws + off_i);
     int l = 0;
     h->nstages = 0;
-    RefView rv{rs.R, rs.m, rs.d, rs.R_lp, rs.kp, rs.rmax2};
+    RefView rv{rs.R, rs.m, rs.d, rs.R_lp, rs.kp, rs.rmax2, rs.centre};
     s = enqueue_search(h, sp, rv, rs.R, n, k + 1, metric, dtmp, itmp, ws, &h->counters->fallback_count,
                        st, &l, false, true);
     if (s != KNN_OK) return s;

@@ -352,14 +352,19 @@ struct HitScale {
 };
 
 // Operand pairs (rows of up to kPairMaxD coordinates): both copies of a search
-// in one launch, the queries' squared norms, and its two queue counters
-// cleared.  R_lp holds whole tiles, pair_tiles(m) of them.
+// in one launch, the queries' squared norms (less twice their remainders), and
+// its two queue counters cleared.  R_lp holds whole tiles, pair_tiles(m) of them.
 constexpr int64_t kPairTile = 256;
 inline int64_t pair_tiles(int64_t m) { return (m + kPairTile - 1) / kPairTile; }
 bool pair_rows_fit(int32_t d);
-cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* Q, int64_t n, int32_t d,
-                                int32_t kp, void* R_lp, void* Q_lp, float* qnorm, int32_t* count0,
-                                int32_t* count1, cudaStream_t st, int* launches);
+cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* centre, const float* Q,
+                                int64_t n, int32_t d, int32_t kp, void* R_lp, void* Q_lp,
+                                float* qnorm, int32_t* count0, int32_t* count1, cudaStream_t st,
+                                int* launches);
+// The centre [d] that the pairs' coordinates are taken relative to: once per
+// reference set.
+cudaError_t launch_centre(const float* R, int64_t m, int32_t d, float* centre, cudaStream_t st,
+                          int* launches);
 
 // Reference copy [r, -||r||^2/2 (hi, lo), 1, 1, 0..], float32 norms and their maximum.
 cudaError_t launch_prepare_ref(const float* R, int64_t m, int32_t d, int32_t kp, int prec,

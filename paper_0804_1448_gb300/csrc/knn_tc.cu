@@ -381,9 +381,17 @@ cudaError_t launch_prepare_ref(const float* R, int64_t m, int32_t d, int32_t kp,
     return cudaGetLastError();
 }
 
-cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* Q, int64_t n, int32_t d,
-                                int32_t kp, void* R_lp, void* Q_lp, float* qnorm, int32_t* count0,
-                                int32_t* count1, cudaStream_t st, int* launches) {
+cudaError_t launch_centre(const float* R, int64_t m, int32_t d, float* centre, cudaStream_t st,
+                          int* launches) {
+    centre_kernel<<<(d + 63) / 64, 64, 0, st>>>(R, m, d, centre);
+    if (launches) ++*launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* centre, const float* Q,
+                                int64_t n, int32_t d, int32_t kp, void* R_lp, void* Q_lp,
+                                float* qnorm, int32_t* count0, int32_t* count1, cudaStream_t st,
+                                int* launches) {
     const int64_t tiles = pair_tiles(m);
     const int rpw = kPairRows * (d <= 16 ? 4 : (d <= 32 ? 2 : 1));   // rows per warp
     const int64_t ref_warps = tiles * kTileN / rpw;
@@ -394,7 +402,7 @@ cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* Q, int64
                 : d <= 64  ? prepare_pair_kernel<32, 1>
                 : d <= 128 ? prepare_pair_kernel<32, 2>
                            : prepare_pair_kernel<32, 3>;
-    kern<<<grid, 256, 0, st>>>(R, m, tiles, Q, n, d, kp, static_cast<uint32_t*>(R_lp),
+    kern<<<grid, 256, 0, st>>>(R, m, tiles, centre, Q, n, d, kp, static_cast<uint32_t*>(R_lp),
                                static_cast<uint32_t*>(Q_lp), qnorm, ref_warps, count0, count1);
     if (launches) ++*launches;
     return cudaGetLastError();

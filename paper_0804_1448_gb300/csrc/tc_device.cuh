@@ -751,10 +751,13 @@ __device__ __forceinline__ void put(void* row, int t, float v) {
 // is made of exact float32 distances either way (its error against float64 is
 // the same to the digit).
 //
-// x = h + l + e with h = bf16(x), l = bf16(x - h), |l| <= 2^-8 |x| and
-// |e| <= 2^-16 |x|.  The three products h.h + l.h + h.l on the tensor cores
-// leave out at most 3.01 * 2^-16 sum |q_t r_t| of q.r, and sum |q_t r_t| <=
-// (n_q + n_r) / 2 with n the squared norms: 1.505 * 2^-16 (n_q + n_r).
+// x = h + r with h = bf16(x), r = l + e with l = bf16(r), both differences exact
+// in float32 and |e| <= 2^-8 |r|.  The three products h.h + l.h + h.l on the
+// tensor cores leave l.l + e_q.r + (q - e_q).e_r out of q.r.  With |a.b| <= (|a|^2 +
+// |b|^2) / 2 and |e.x| <= (A |e|^2 + |x|^2 / A) / 2, A = 2^17, that is at most w_q +
+// w_r + 2^-18 (1 + 2^-15) (n_q + n_r), where n is a row's squared norm and w = 1.504
+// |r|^2 comes from its own coordinates: 0.23 * 2^-16 n for those of ordinary
+// points, 1.5 * 2^-16 n where every one is as far from its upper word as it gets.
 //
 // Row layout (elements): h words [0, 16 hs), l words [16 hs, 32 hs), hs =
 // ceil(d / 16); five more words -- the reference's norm in three parts
@@ -772,7 +775,7 @@ __host__ __device__ constexpr int pair_ksteps(int d) {
 }
 
 // Error bound of acc = q'.r' - n_r/2 + t as the tensor cores return it, as
-// eq n_q + er n_r + acc |t|.  Besides the words left out: each of the
+// w_q + w_r + eq n_q + er n_r + acc |t|.  Besides the words left out: each of the
 // 3 hs MMA steps (and the one of the extra words, if any) adds 16 exact products
 // to the accumulator, with an error of at most 17 * 2^-24 of the largest among
 // the products and the sums before and after, which is at most 1.02 (n_q +
@@ -785,11 +788,13 @@ __host__ __device__ constexpr int pair_ksteps(int d) {
 struct PairSlack {
     float eq, er, acc;
 };
+// w over |r|^2, with 0.1% for the rounding of the sum.
+constexpr float kPairLeft = 1.506f;
 __host__ __device__ inline PairSlack pair_slack(int d) {
     constexpr float u = 5.9604644775390625e-8f;   // 2^-24
     PairSlack s;
     s.acc = 17.f * u * static_cast<float>(3 * pair_hsteps(d) + (pair_aug_inside(d) ? 0 : 1));
-    const float common = 1.505f * 256.f * u + static_cast<float>(d + 16) * u;
+    const float common = 64.01f * u + static_cast<float>(d + 16) * u;
     s.eq = common + 0.51f * s.acc;
     s.er = common + 1.02f * s.acc;
     return s;
@@ -799,6 +804,38 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
 }
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// The centre of a reference set: every coordinate's median over kCentreRows
+// evenly spaced rows (fewer in a smaller set), a thread per coordinate.  The
+// pairs' slack grows with the squared distances from it, so it must not be a
+// row that lies far out: with row 0 as the centre and row 0 moved by 30, no query
+// of a uniform set could be certified.  It also halves the slack of a set whose
+// rows lie all around: 10% of the queries of a Gaussian mixture (m = 1 million,
+// d = 128, k = 100) were uncertified about row 0.  Medians of coordinates that
+// are not finite become 0.
+constexpr int kCentreRows = 33;
+__global__ void centre_kernel(const float* __restrict__ R, int64_t m, int32_t d,
+                              float* __restrict__ centre) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= d) return;
+    const int cnt = static_cast<int>(min(m, static_cast<int64_t>(kCentreRows)));
+    uint32_t v[kCentreRows];
+#pragma unroll
+    for (int i = 0; i < kCentreRows; ++i)
+        v[i] = i < cnt ? ord_f32(R[(2 * i + 1) * m / (2 * cnt) * d + t]) : 0xffffffffu;
+    uint32_t med = 0;
+#pragma unroll
+    for (int i = 0; i < kCentreRows; ++i) {
+        int below = 0;
+#pragma unroll
+        for (int j = 0; j < kCentreRows; ++j) below += (v[j] < v[i] || (v[j] == v[i] && j < i)) ? 1 : 0;
+        if (below == cnt / 2) med = v[i];
+    }
+    const float c = unord_f32(med);
+    centre[t] = fabsf(c) < __builtin_huge_valf() ? c : 0.f;
+}
 
 constexpr int kPairRows = 4;   // rows per group of lanes
 constexpr int kPairMaxD = 192;
@@ -806,9 +843,9 @@ constexpr int kPairMaxD = 192;
 // Operand rows of a search on pairs, references and queries in one launch: a
 // row per LANES lanes (8 up to d = 16, 16 up to 32, else a whole warp, NJ
 // coordinate pairs a lane), kPairRows rows at a time; warps below ref_warps take
-// consecutive rows of the reference copy, the others queries.  Coordinates are taken relative to the set's first
-// reference, so the slack follows the data's spread, not its offset from the
-// origin.  Row p of the copy, column c of tile g, holds reference
+// consecutive rows of the reference copy, the others queries.  Coordinates are
+// taken relative to a centre of the set (centre_kernel), so the slack follows the
+// data's spread, not its offset from the origin.  Row p of the copy, column c of tile g, holds reference
 // ((c mod 64) 4 + c / 64) T + g: every tile is an evenly spaced sample of the
 // whole set, and neighbours in storage order go to different column groups, so
 // a set stored cluster by cluster gives the pilot's sample and the hit lists
@@ -820,8 +857,10 @@ constexpr int kPairMaxD = 192;
 // per row whatever d, with room for 192 coordinates: 19 us for
 // the self-join of 20000 points, d = 3; 23 against 27 at n = m = 38400, d = 96.)  It also clears the search's two queue counters.
 template <int LANES, int NJ>
-__global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int64_t tiles,
-                                    const float* __restrict__ Q, int64_t n, int32_t d, int32_t kp,
+__global__ void __launch_bounds__(256, LANES > 8 && NJ == 1 ? 5 : 4)
+prepare_pair_kernel(const float* __restrict__ R, int64_t m, int64_t tiles,
+                                    const float* __restrict__ centre, const float* __restrict__ Q,
+                                    int64_t n, int32_t d, int32_t kp,
                                     uint32_t* __restrict__ R_lp, uint32_t* __restrict__ Q_lp,
                                     float* __restrict__ qnorm, int64_t ref_warps,
                                     int32_t* __restrict__ count0, int32_t* __restrict__ count1) {
@@ -852,38 +891,54 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
         }
     }
     float xv[RW][NJ][2];
+    if ((d & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 7) == 0) {   // whole pairs, 8-byte aligned
 #pragma unroll
-    for (int u = 0; u < RW; ++u)
+        for (int u = 0; u < RW; ++u)
 #pragma unroll
-        for (int j = 0; j < NJ; ++j)
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const int t = 2 * lane + 2 * LANES * j + b;
-                xv[u][j][b] = (src[u] >= 0 && t < d) ? __ldg(X + src[u] * d + t) : 0.f;
+            for (int j = 0; j < NJ; ++j) {
+                const int t = 2 * lane + 2 * LANES * j;
+                float2 v = make_float2(0.f, 0.f);
+                if (src[u] >= 0 && t < d) v = __ldg(reinterpret_cast<const float2*>(X + src[u] * d + t));
+                xv[u][j][0] = v.x;
+                xv[u][j][1] = v.y;
             }
-    float nr[RW];
+    } else {
 #pragma unroll
-    for (int u = 0; u < RW; ++u) nr[u] = 0.f;
+        for (int u = 0; u < RW; ++u)
 #pragma unroll
-    for (int j = 0; j < NJ; ++j)
+            for (int j = 0; j < NJ; ++j)
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int t = 2 * lane + 2 * LANES * j + b;
-            if (t < d) {
-                const float c = __ldg(R + t);
-#pragma unroll
-                for (int u = 0; u < RW; ++u) {
-                    if (src[u] >= 0) {
-                        xv[u][j][b] -= c;
-                        nr[u] = fmaf(xv[u][j][b], xv[u][j][b], nr[u]);
-                    }
+                for (int b = 0; b < 2; ++b) {
+                    const int t = 2 * lane + 2 * LANES * j + b;
+                    xv[u][j][b] = (src[u] >= 0 && t < d) ? __ldg(X + src[u] * d + t) : 0.f;
                 }
-            }
+    }
+    float nr[RW], left[RW];            // |x|^2, |r|^2
+    uint32_t hw[RW][NJ], lw[RW][NJ];   // the coordinate pairs' h and l words
+#pragma unroll
+    for (int u = 0; u < RW; ++u) nr[u] = left[u] = 0.f;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int t = 2 * lane + 2 * LANES * j;
+        const float c0 = t < d ? __ldg(centre + t) : 0.f, c1 = t + 1 < d ? __ldg(centre + t + 1) : 0.f;
+#pragma unroll
+        for (int u = 0; u < RW; ++u) {
+            const float x0 = src[u] >= 0 ? xv[u][j][0] - c0 : 0.f;
+            const float x1 = src[u] >= 0 ? xv[u][j][1] - c1 : 0.f;
+            nr[u] = fmaf(x0, x0, fmaf(x1, x1, nr[u]));
+            hw[u][j] = bf16x2_bits(x0, x1);
+            const float r0 = x0 - bf16_lo(hw[u][j]), r1 = x1 - bf16_hi(hw[u][j]);
+            lw[u][j] = bf16x2_bits(r0, r1);
+            left[u] = fmaf(r0, r0, fmaf(r1, r1, left[u]));
         }
+    }
 #pragma unroll
     for (int o = LANES / 2; o > 0; o >>= 1)
 #pragma unroll
-        for (int u = 0; u < RW; ++u) nr[u] += __shfl_xor_sync(0xffffffffu, nr[u], o);
+        for (int u = 0; u < RW; ++u) {
+            nr[u] += __shfl_xor_sync(0xffffffffu, nr[u], o);
+            left[u] += __shfl_xor_sync(0xffffffffu, left[u], o);
+        }
     const int hs = pair_hsteps(d);
     const bool inside = pair_aug_inside(d);
     const float half_er = 0.5f - pair_slack(d).er;   // -(1/2 - er) n_r: er n_r of slack on acc
@@ -893,8 +948,8 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
         if (p >= rows) break;
         float aug[kPairAug];
         if (ref) {
-            // -(1 - 2 er) n_r / 2 in three parts
-            const float v = src[u] >= 0 ? -half_er * nr[u] : -3e38f;
+            // -(1 - 2 er) n_r / 2 + w_r in three parts
+            const float v = src[u] >= 0 ? fmaf(-half_er, nr[u], kPairLeft * left[u]) : -3e38f;
             aug[0] = lowp_round<kBF16>(v);
             aug[1] = lowp_round<kBF16>(v - aug[0]);
             aug[2] = (v - aug[0]) - aug[1];
@@ -903,7 +958,7 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
         } else {
             aug[0] = aug[1] = aug[2] = 1.f;
             aug[3] = aug[4] = 0.f;
-            if (lane == 0) qnorm[p] = nr[u];
+            if (lane == 0) qnorm[p] = fmaf(-2.f * kPairLeft, left[u], nr[u]);
         }
         auto aug_at = [&](int i) {   // the i-th extra word, 0 outside
             float v = 0.f;
@@ -916,14 +971,10 @@ __global__ void prepare_pair_kernel(const float* __restrict__ R, int64_t m, int6
         for (int j = 0; j < NJ; ++j) {
             const int t = 2 * lane + 2 * LANES * j;
             if (t >= 16 * hs) break;
-            const float x0 = xv[u][j][0], x1 = xv[u][j][1];
-            float h0 = lowp_round<kBF16>(x0), h1 = lowp_round<kBF16>(x1);
-            row[8 * hs + t / 2] = bf16x2_bits(t < d ? x0 - h0 : 0.f, t + 1 < d ? x1 - h1 : 0.f);
-            if (inside) {
-                if (t >= d) h0 = aug_at(t - d);
-                if (t + 1 >= d) h1 = aug_at(t + 1 - d);
-            }
-            row[t / 2] = bf16x2_bits(h0, h1);
+            row[8 * hs + t / 2] = lw[u][j];
+            row[t / 2] = inside && t + 1 >= d
+                             ? bf16x2_bits(t < d ? bf16_lo(hw[u][j]) : aug_at(t - d), aug_at(t + 1 - d))
+                             : hw[u][j];
         }
         for (int e = 2 * lane; e < kp - 32 * hs; e += 2 * LANES)
             row[16 * hs + e / 2] =
@@ -1136,8 +1187,8 @@ __device__ __forceinline__ uint32_t order_statistic(const uint32_t* __restrict__
     return nvalid >= cprime ? prefix : least;   // fewer than cprime groups: the weakest
 }
 
-// Operand pairs (PREC = kPair): qscale[q] holds the query's squared norm n_q;
-// in its place goes the bound that certifies the query's answer.  With the
+// Operand pairs (PREC = kPair): qscale[q] holds the query's squared norm n_q less
+// 2 w_q; in its place goes the bound that certifies the query's answer.  With the
 // norm words slack of the reference folded in (pair_slack), every reference
 // has ||q - r||^2 >= bound - 2 acc, so those that fail the filter are at least
 // `bound` away.  A query whose norm is not finite or above 1e36 (where float32
@@ -1174,10 +1225,10 @@ __device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gma
             put<kBF16>(row, at + 1, lo);
             const PairSlack ps = pair_slack(d);
             const float t = hi + lo;
-            // float32 rounding of the four operations here: 8 and 16 units of
-            // 2^-24; squares that underflow: 1e-33
+            // float32 rounding of the operations here and of n_q - 2 w_q: 10 and 16
+            // units of 2^-24; squares that underflow: 1e-33
             constexpr float u = 5.9604644775390625e-8f;
-            const float b = nq2 * (1.f - 2.f * ps.eq - 8.f * u) + 2.f * t -
+            const float b = nq2 * (1.f - 2.f * ps.eq - 10.f * u) + 2.f * t -
                             (2.f * ps.acc + 16.f * u) * fabsf(t) - 1e-33f;
             qscale[q] = nq2 <= 1e36f ? b : __int_as_float(0xff800000);
         }

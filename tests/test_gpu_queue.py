@@ -66,3 +66,54 @@ def test_short_queues_of_a_large_set_take_the_select(knn, m, direct):
         assert st["fallback_queries"] > 8
     else:
         assert st["fallback_queries"] == 0
+
+
+@pytest.mark.parametrize("where", ["first", "middle", "huge", "nan"])
+@pytest.mark.parametrize("d", [8, 32, 96])
+def test_outliers_do_not_move_the_centre(knn, d, where):
+    """A row far from all others, or one that is no point at all, wherever it is
+    stored: the filter still certifies (what 20 queries among 20000 references
+    leave uncertified goes to the exact fallback)."""
+    R = inputs.uniform(20000, d, seed=91)
+    Q = inputs.uniform(20, d, seed=92)
+    if where == "first":
+        R[0] += np.float32(30.0)
+    elif where == "middle":
+        R[10000:10010] -= np.float32(1000.0)
+    elif where == "huge":
+        R[0] = np.float32(1e30)
+    else:
+        R[0] = np.nan
+    if where == "nan":   # the oracle has no order for it: the other rows, moved up by one
+        import torch
+        ix = knn.Index(0, "fp32")
+        ix.set_reference(torch.from_numpy(R).cuda())
+        dist, idx = ix.search(torch.from_numpy(Q).cuda(), 10)
+        ix.sync()
+        st = ix.stats()
+        ix.close()
+        o_dist, o_idx = oracle.knn(R[1:], Q, parity.oracle_k(10, 19999), "l2")
+        parity.compare(dist.cpu().numpy(), idx.cpu().numpy() - 1, o_dist, o_idx, 10, 19999)
+    else:
+        st = check(knn, R, Q, 10)
+    assert st["fallback_queries"] == 0
+
+
+def test_centre_of_a_whitened_set(knn):
+    """Mahalanobis searches run on whitened rows, which have a centre of their own."""
+    import torch
+    d = 24
+    R = inputs.uniform(20000, d, seed=93) + np.float32(50.0)
+    R[0] += np.float32(30.0)
+    Q = inputs.uniform(20, d, seed=94) + np.float32(50.0)
+    M = np.diag(np.linspace(1.0, 4.0, d))
+    ix = knn.Index(0, "fp32")
+    ix.set_reference(torch.from_numpy(R).cuda())
+    ix.set_mahalanobis(M)
+    dist, idx = ix.search(torch.from_numpy(Q).cuda(), 10, "mahalanobis")
+    ix.sync()
+    st = ix.stats()
+    ix.close()
+    o_dist, o_idx = oracle.knn_mahalanobis(R, Q, M, parity.oracle_k(10, 20000))
+    parity.compare(dist.cpu().numpy(), idx.cpu().numpy(), o_dist, o_idx, 10, 20000)
+    assert st["fallback_queries"] == 0
