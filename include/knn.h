@@ -192,7 +192,8 @@ typedef struct {
     int64_t chunk;              /* references per split */
                                 /* float32 Euclidean searches with k_blocks > 0 run a
                                    tensor-core filter on pairs of bf16 words first, and the
-                                   fields from k_blocks to list_capacity are that filter's;
+                                   candidates and the fields from k_blocks to
+                                   list_capacity are that filter's;
                                    splits and chunk are the select's, which takes the
                                    queries the filter cannot certify */
     int32_t k_blocks;           /* tensor cores: 128-byte K blocks per operand row */

@@ -332,6 +332,7 @@ struct SearchPlan {
     int prec = 0;
     int kp = 0;
     int c = 0;
+    int fc = 0;              // pair: candidates the filter keeps (c: the select's)
     int S = 1;
     int64_t chunk = 0;
     TcPlan plan{};
@@ -343,14 +344,23 @@ struct SearchPlan {
     size_t bytes = 0;
 };
 
-// The operand-pair filter of a float32 Euclidean search (c candidates), when
-// its rows fit the tensor-core tile (d up to 187) and its pilot runs.  It is
-// the faster form at every size above the small-set select's: one query among
-// 5000 references, d = 8, 52 us against 97 us with the CUDA-core select; 64
-// among 2 million, d = 96, 0.80 ms against 1.96; 4000 among 100000, d = 128,
-// 0.44 ms against 3.90; n = m = 38400, d = 96, 0.86 ms against 8.57.
-bool plan_pair(int64_t n, int64_t m, int32_t d, int32_t c, int sm_share, SearchPlan* p) {
-    if (!pair_rows_fit(d) || 2 * c + 32 > finalize_max_pool()) return false;
+// The operand-pair filter of a float32 Euclidean search whose select keeps c
+// candidates, when its rows fit the tensor-core tile (d up to 187), its pilot
+// runs and its answers can be expected to be certified with up to four times as
+// many (pair_candidates).  There it is the faster form at every size above the
+// small-set select's: one query among 5000 references, d = 8, 30 us against 97 us
+// with the CUDA-core select; 64 among 2 million, d = 96, 0.80 ms against 1.96; 4000
+// among 100000, d = 128, 0.44 ms against 3.90; n = m = 38400, d = 96, 0.86 ms
+// against 8.57.  Where the points are too dense for it (k = 10: from m = 6300 on
+// at d = 1, 690000 at d = 2, 54 million at d = 3) it would filter, certify next to
+// nothing and take the select all the same: n = 300, m = 4 million, d = 2, 3.1 ms
+// against 2.5, and n = 16 through the exact fallback 66 ms against 0.9.
+bool plan_pair(int64_t n, int64_t m, int32_t d, int32_t k, int sm_share, SearchPlan* p) {
+    if (!pair_rows_fit(d)) return false;
+    const int64_t need = pair_candidates(m, d, k);
+    if (need > 4LL * p->c) return false;
+    const int32_t c = std::max(p->c, static_cast<int32_t>(need));
+    if (2 * c + 32 > finalize_max_pool()) return false;
     const int kp = tc_padded_dim(d, kPair);
     const TcPlan t = tc_plan(n, pair_tiles(m) * kPairTile, d, kp, kPair, c, sm_share);
     if (t.stages == 0 || !t.raw || !t.pilot) return false;
@@ -358,6 +368,7 @@ bool plan_pair(int64_t n, int64_t m, int32_t d, int32_t c, int sm_share, SearchP
     p->plan.m_set = m;
     p->prec = kPair;
     p->kp = kp;
+    p->fc = c;
     return true;
 }
 
@@ -417,7 +428,7 @@ knn_status plan_search_md(const knn_ctx* h, int64_t m, int32_t d, int precision,
         if (static_cast<int64_t>(S) * p.c > finalize_max_pool()) return KNN_ERR_UNSUPPORTED;
         p.S = S;
         p.chunk = chunk;
-        p.pair = allow_filter && metric == KNN_L2 && plan_pair(n, m, d, p.c, sm_share, &p);
+        p.pair = allow_filter && metric == KNN_L2 && plan_pair(n, m, d, k, sm_share, &p);
         if (allow_filter && metric != KNN_L2 && 2 * p.c + 32 <= finalize_max_pool()) {
             p.dplan = diff_plan(n, m, d, p.c, sm_share);
             p.diff = p.dplan.pilot;
@@ -586,7 +597,7 @@ knn_status enqueue_search(knn_ctx* h, const SearchPlan& sp, const RefView& rv, c
         fa.hits.counts = counts;
         fa.hits.S = plan.groups * plan.S;   // one list per (split, epilogue column group)
         fa.hits.cap = plan.cap;
-        fa.hits.c = c;
+        fa.hits.c = sp.pair ? sp.fc : c;
         fa.hits.bound = sp.pair ? qs.qscale : nullptr;
         fa.cand.exact = 0;
         fa.cand.S = 1;
@@ -1592,7 +1603,7 @@ knn_status knn_explain_plan(int64_t n, int64_t m, int32_t d, int32_t k, knn_metr
     if (s != KNN_OK) return s;
     knn_plan o{};
     o.tensor_cores = sp.tensor ? 1 : 0;
-    o.candidates = sp.c;
+    o.candidates = sp.pair ? sp.fc : sp.c;
     o.splits = sp.S;
     o.chunk = sp.chunk;
     if (sp.tensor || sp.pair) {

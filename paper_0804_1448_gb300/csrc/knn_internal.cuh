@@ -357,6 +357,9 @@ struct HitScale {
 constexpr int64_t kPairTile = 256;
 inline int64_t pair_tiles(int64_t m) { return (m + kPairTile - 1) / kPairTile; }
 bool pair_rows_fit(int32_t d);
+// How many candidates the filter must keep for the k nearest of m references
+// to be certified (more than m: hopeless).
+int64_t pair_candidates(int64_t m, int32_t d, int32_t k);
 cudaError_t launch_prepare_pair(const float* R, int64_t m, const float* centre, const float* Q,
                                 int64_t n, int32_t d, int32_t kp, void* R_lp, void* Q_lp,
                                 float* qnorm, int32_t* count0, int32_t* count1, cudaStream_t st,

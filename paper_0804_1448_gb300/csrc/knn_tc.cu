@@ -214,6 +214,30 @@ cudaError_t launch_mma_probe(const float* A, const float* B, int32_t steps, floa
 
 bool pair_rows_fit(int32_t d) { return d >= 1 && d <= kPairMaxD; }
 
+// An answer is certified when the nearest reference that was not kept is further
+// than the k-th by the bound's slack: the candidates must reach as far as that.
+// For points uniform in a cube of side 1, d / 12 from their centre on average
+// (squared), the slack is s = d / 12 (2 eq + 2 er + a), rows' remainders added, and
+// the k-th distance r^2 = (k / (m V_d))^(2 / d), V_d the volume of the unit ball, so
+// k ((1 + s / r^2)^(d / 2) - 1) = L references are expected in between.  2.5 L + 4
+// sqrt(L) + 4 covers the spread of their number and the corners of the cube,
+// whose rows lie further out (simulated over d = 1 to 12, m = 5000 to 4 million, k =
+// 1 to 100, with 2.5 times this slack: a query in a thousand needed more).  L is
+// below 1 from d = 4 on, and large where the points are dense on the scale of
+// their spread: k = 10, 0.2 at d = 3, m = 100000, 2.5 at m = 4 million; 2.4 at d = 2,
+// m = 100000, 24 at m = 1 million; 12 at d = 1, m = 5000.
+int64_t pair_candidates(int64_t m, int32_t d, int32_t k) {
+    constexpr double kPi = 3.14159265358979323846;
+    const PairSlack ps = pair_slack(d);
+    const double left = 0.23 / 65536.0;   // a row's own remainder, of its norm (uniform points)
+    const double s = d / 12.0 * (2.0 * ps.eq + 2.0 * ps.er + 4.0 * left + ps.acc);
+    const double log_v = 0.5 * d * std::log(kPi) - std::lgamma(0.5 * d + 1.0);
+    const double r2 = std::exp(2.0 / d * (std::log(static_cast<double>(k) / static_cast<double>(m)) - log_v));
+    const double l = k * std::expm1(0.5 * d * std::log1p(s / r2));
+    const double need = k + std::ceil(2.5 * l + 4.0 * std::sqrt(l) + 4.0);
+    return need <= static_cast<double>(m) ? static_cast<int64_t>(need) : m + 1;
+}
+
 int tc_padded_dim(int32_t d, int prec) {
     if (prec == kPair) return pair_ksteps(d) * 16;
     const int step = (prec == kTF32) ? 8 : 16;   // whole 32-byte MMA K steps per row
