@@ -1191,8 +1191,9 @@ __device__ __forceinline__ uint32_t order_statistic(const uint32_t* __restrict__
 // 2 w_q; in its place goes the bound that certifies the query's answer.  With the
 // norm words slack of the reference folded in (pair_slack), every reference
 // has ||q - r||^2 >= bound - 2 acc, so those that fail the filter are at least
-// `bound` away.  A query whose norm is not finite or above 1e36 (where float32
-// squares overflow) gets -inf: it is never certified.
+// `bound` away.  A query whose norm is not finite or above 1e36, or whose
+// threshold is above 1e37 (where float32 squares, or twice the threshold, overflow),
+// gets -inf: it is never certified.
 template <int PREC, int VPL>
 __device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gmax, int64_t q,
                                                 int32_t G, int32_t cprime, int32_t d, int32_t kp,
@@ -1230,7 +1231,7 @@ __device__ __forceinline__ void threshold_query(const uint32_t* __restrict__ gma
             constexpr float u = 5.9604644775390625e-8f;
             const float b = nq2 * (1.f - 2.f * ps.eq - 10.f * u) + 2.f * t -
                             (2.f * ps.acc + 16.f * u) * fabsf(t) - 1e-33f;
-            qscale[q] = nq2 <= 1e36f ? b : __int_as_float(0xff800000);
+            qscale[q] = nq2 <= 1e36f && fabsf(t) <= 1e37f ? b : __int_as_float(0xff800000);
         }
         return;
     }

@@ -129,3 +129,28 @@ def test_dense_points(knn, n, m, d, k):
     st = check(knn, inputs.uniform(m, d, seed=95), inputs.uniform(n, d, seed=96), k,
                rows=np.arange(0, n, max(1, n // 32)))
     assert st["fallback_queries"] <= n // 100
+
+
+def test_bound_near_the_float32_limit(knn):
+    """Squared distances within 3e-5 of the largest float32, queries at the
+    centre: the threshold passes half that limit, and twice it must not become a
+    bound of +inf, which would certify whatever the cut left.  Each far row has
+    its length in two coordinates with large remainders, which the filter's
+    slack counts as nearness; the ten nearest have theirs in one, with none."""
+    d, m = 16, 4352
+    g = np.random.default_rng(21)
+    R = np.zeros((m, d))
+    pair = g.integers(0, d // 2, m)
+    top = 3.40281e38
+    a = np.float32(1.0 + 2.0 ** -8 - 2.0 ** -17) * 2.0 ** 63          # just past a bf16 half unit
+    b = np.sqrt(top * (1 - 8e-6 * g.random(m)) - a.astype(np.float64) ** 2)
+    rows = np.arange(m)
+    R[rows, 2 * pair] = g.choice([-1.0, 1.0], m) * a
+    R[rows, 2 * pair + 1] = g.choice([-1.0, 1.0], m) * b
+    near = 100 + 400 * np.arange(10)
+    R[near] = 0
+    R[near, 2 * pair[near]] = 2.0 ** 64 * (1 - 8e-6 - 4e-7 * np.arange(10))
+    R = R.astype(np.float32)
+    assert np.all(np.isfinite((R * R).sum(1, dtype=np.float32)))
+    Q = np.zeros((16, d), np.float32)
+    check(knn, R, Q, 10)
