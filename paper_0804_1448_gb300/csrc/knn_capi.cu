@@ -78,6 +78,8 @@ struct knn_ctx {
     // workspace (grown on demand, or reserved up front with knn_reserve)
     unsigned char* ws = nullptr;
     size_t ws_bytes = 0;
+    // the last growth that the device refused, and the memory it had then (0: none)
+    size_t refused = 0, refused_have = 0;
 
     Counters* counters = nullptr;  // device
     int32_t* flag_host = nullptr;  // pinned host word: the error flag as a host-buffer search ends
@@ -147,9 +149,11 @@ knn_status cuda_fail(knn_ctx* h, cudaError_t err, const char* what) {
         if (err__ != cudaSuccess) return cuda_fail((h), err__, #call); \
     } while (0)
 
-bool fault_inject_oom() {
+// KNN_FAULT_INJECT_OOM: 1 refuses every growth of a workspace; a larger number
+// is the device memory that workspaces are to find, in bytes.
+long long fault_inject_oom() {
     const char* v = std::getenv("KNN_FAULT_INJECT_OOM");
-    return v && v[0] == '1';
+    return v ? std::atoll(v) : 0;
 }
 
 void drop_graphs(knn_ctx* h) {
@@ -160,10 +164,20 @@ void drop_graphs(knn_ctx* h) {
     h->graphs.clear();
 }
 
+// The device memory that a workspace in place of the one held could find.
+size_t memory_to_have(const knn_ctx* h) {
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess) (void)cudaGetLastError();
+    const long long most = fault_inject_oom();
+    const size_t have = free + h->ws_bytes;
+    return most > 1 ? std::min(have, static_cast<size_t>(most)) : have;
+}
+
 // Make sure the handle's workspace holds at least `bytes`.
 knn_status ensure_workspace(knn_ctx* h, size_t bytes) {
     if (bytes <= h->ws_bytes) return KNN_OK;
-    if (fault_inject_oom()) {
+    const long long most = fault_inject_oom();
+    if (most == 1) {
         h->last_error = "workspace allocation refused (KNN_FAULT_INJECT_OOM=1)";
         return KNN_ERR_OOM;
     }
@@ -176,15 +190,25 @@ knn_status ensure_workspace(knn_ctx* h, size_t bytes) {
     if (h->ws) KNN_CUDA(h, cudaFree(h->ws));
     h->ws = nullptr;
     h->ws_bytes = 0;
+    auto get = [&](size_t n) {
+        return most > 1 && n > static_cast<size_t>(most) ? cudaErrorMemoryAllocation : cudaMalloc(&h->ws, n);
+    };
     const size_t grow = bytes + bytes / 4;
-    cudaError_t err = cudaMalloc(&h->ws, grow);
+    cudaError_t err = get(grow);
     if (err != cudaSuccess) {
-        err = cudaMalloc(&h->ws, bytes);
-        if (err != cudaSuccess) return cuda_fail(h, err, "cudaMalloc(workspace)");
+        (void)cudaGetLastError();
+        err = get(bytes);
+        if (err != cudaSuccess) {
+            const knn_status s = cuda_fail(h, err, "cudaMalloc(workspace)");
+            h->refused = bytes;
+            h->refused_have = memory_to_have(h);
+            return s;
+        }
         h->ws_bytes = bytes;
     } else {
         h->ws_bytes = grow;
     }
+    if (bytes >= h->refused) h->refused = 0;
     return KNN_OK;
 }
 
@@ -504,6 +528,15 @@ knn_status plan_search(const knn_ctx* h, int64_t n, int32_t k, knn_metric metric
                           h->num_sms, sp, 64LL << 20, allow_filter);
 }
 
+// Whether a workspace of `bytes`, more than the one held, may be tried for: a try
+// that fails costs a device-wide synchronisation, the batch graphs and the
+// workspace held, in every search again.  So there must be memory for it, and
+// more than at the last refusal of no more bytes.
+bool may_grow(const knn_ctx* h, size_t bytes) {
+    const size_t have = memory_to_have(h);
+    return have >= bytes && !(h->refused > 0 && bytes >= h->refused && have <= h->refused_have);
+}
+
 // Plan a search on st and hold its workspace, `extra` bytes after the plan's
 // own included.  A float32 search whose filter's scratch cannot be had --
 // no memory, or a capturing stream and a workspace that would have to grow --
@@ -515,7 +548,9 @@ knn_status plan_and_hold(knn_ctx* h, int64_t n, int32_t k, knn_metric metric, in
     if (sp->filtered() && sp->bytes + extra > h->ws_bytes) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         KNN_CUDA(h, cudaStreamIsCapturing(st, &cap));
-        s = cap == cudaStreamCaptureStatusNone ? ensure_workspace(h, sp->bytes + extra) : KNN_ERR_OOM;
+        s = cap == cudaStreamCaptureStatusNone && may_grow(h, sp->bytes + extra)
+                ? ensure_workspace(h, sp->bytes + extra)
+                : KNN_ERR_OOM;
         if (s != KNN_ERR_OOM) return s;
         s = plan_search(h, n, k, metric, io_on_device, sp, false);
         if (s != KNN_OK) return s;
