@@ -154,3 +154,13 @@ def test_bound_near_the_float32_limit(knn):
     assert np.all(np.isfinite((R * R).sum(1, dtype=np.float32)))
     Q = np.zeros((16, d), np.float32)
     check(knn, R, Q, 10)
+
+
+@pytest.mark.parametrize("n,left", [(8192, 150), (9000, 400)])
+def test_queue_of_a_large_search(knn, n, left):
+    """Part of 8192 or more queries left over: the select of 128 queries a CTA
+    over a queue that fills no whole number of them.  It certifies most, though
+    with few splits its own margin of 8 candidates is narrow here."""
+    R, Q = ladders(60000, n, left)
+    st = check(knn, R, Q, 10)
+    assert st["fallback_queries"] < left // 2
