@@ -348,9 +348,18 @@ knn_status knn_create_shared(knn_handle* out, knn_handle src, const knn_options*
  * io_on_device, ...) needs with h's current reference set and precision
  * (written to *bytes; 0 for n = 0).  Nothing is allocated or launched.  With
  * knn_reserve, this lets a caller admit work by memory and keep allocation
- * out of the search path.  (A float32 Euclidean search of a large set includes
- * a copy of the set split into bf16 pairs, about as large as the set; under a
- * workspace_limit too small for it, it plans without.)
+ * out of the search path.
+ * A float32 search of more than 4096 references filters them first, and that
+ * needs more than the select it falls back on: hit lists (8 bytes an entry, a few
+ * hundred to a few thousand entries a query) and pilot maxima (up to 8 KB a
+ * query); in the Euclidean distance also a copy of the set in pairs of bf16 words,
+ * 4 bytes a coordinate with rows padded to 16 coordinates (64 bytes a row at d =
+ * 11 and below, 2.7 times the set at d = 6, 416 bytes or 1.08 times at d = 96).
+ * Where these pass workspace_limit, or 16 GB without one, where the device has no
+ * memory for them, or where the stream is being captured and the workspace held
+ * is too small, the search runs without the filter: the same results, several
+ * times slower on large sets.  Each handle holds its own workspace, also those
+ * that share a reference set, and keeps it until it is destroyed.
  * Errors: as knn_search's argument checks (KNN_ERR_INVALID, KNN_ERR_NOREF,
  * KNN_ERR_UNSUPPORTED); KNN_ERR_INVALID when bytes is NULL.
  */

@@ -807,7 +807,7 @@ knn_status plan_batch(const knn_ctx* h, const knn_instance* inst, int32_t count,
         SearchPlan& sp = bp->sp[i];
         knn_status s = plan_search_md(h, x.m, x.d, h->opt.precision, x.n, x.k,
                                       static_cast<knn_metric>(x.metric), 1, sm_share, &sp,
-                                      4LL << 20, false);   // no reference copy per instance
+                                      4LL << 20, false);   // no filter: no reference copy per instance
         if (s != KNN_OK) return s;
         bp->base[i] = cv.take(sp.bytes);
         bp->fbc[i] = cv.take(sizeof(int32_t));
@@ -1413,7 +1413,9 @@ knn_status knn_search_batch(knn_handle h, const knn_instance* inst, int32_t coun
     cudaStream_t st = cuda_stream ? static_cast<cudaStream_t>(cuda_stream) : h->stream;
 
     if (flags & KNN_BATCH_NO_GRAPH) {
-        // one instance after another on st, each planned as a lone search
+        // one instance after another on st, each planned as a lone search (in
+        // float32 without the filters, whose copies and lists every instance
+        // would need at once)
         BatchPlan bp;
         knn_status s = plan_batch(h, inst, count, h->num_sms, &bp);
         if (s != KNN_OK) return s;

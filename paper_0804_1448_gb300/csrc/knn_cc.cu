@@ -15,8 +15,8 @@
 //
 // Most float32 searches run a filter instead (operand pairs on the tensor
 // cores, knn_tc.cu; Manhattan and Chebyshev, knn_diff.cu).  This form takes
-// what they cannot: rows too long for them, workspace limits, batches, and the
-// queries a filter leaves over (a queue).
+// what they cannot: rows too long for them, points too dense, workspace limits,
+// batches, and the queries a filter leaves over (a queue).
 //
 // Manhattan and Chebyshev distances are formed from coordinate differences in
 // float32, coordinate 0 first (sum_t |q_t - r_t|, max_t |q_t - r_t|).  The

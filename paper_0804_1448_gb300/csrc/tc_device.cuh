@@ -845,25 +845,27 @@ constexpr int kPairMaxD = 192;
 // coordinate pairs a lane), kPairRows rows at a time; warps below ref_warps take
 // consecutive rows of the reference copy, the others queries.  Coordinates are
 // taken relative to a centre of the set (centre_kernel), so the slack follows the
-// data's spread, not its offset from the origin.  Row p of the copy, column c of tile g, holds reference
-// ((c mod 64) 4 + c / 64) T + g: every tile is an evenly spaced sample of the
-// whole set, and neighbours in storage order go to different column groups, so
-// a set stored cluster by cluster gives the pilot's sample and the hit lists
-// the same shares as a shuffled one.  Rows past the set get a norm word no
-// threshold passes.
-// The kernel reads and writes each row once, so memory bounds it; a lane holds
-// two neighbouring coordinates and stores them as one 32-bit word of h and one
-// of l, and all loads of its rows are issued before the first is used.  (A warp
-// per row whatever d, with room for 192 coordinates: 19 us for
-// the self-join of 20000 points, d = 3; 23 against 27 at n = m = 38400, d = 96.)  It also clears the search's two queue counters.
+// data's spread, not its offset from the origin.  Row p of the copy, column c of
+// tile g, holds reference ((c mod 64) 4 + c / 64) T + g: every tile is an evenly
+// spaced sample of the whole set, and neighbours in storage order go to different
+// column groups, so a set stored cluster by cluster gives the pilot's sample and
+// the hit lists the same shares as a shuffled one.  Rows past the set get a norm
+// word no threshold passes.  It also clears the search's two queue counters.
+// The kernel reads and writes each row once, so memory bounds it, and what it
+// reaches of that is a matter of loads in flight (m = 2 million, d = 96: 430 us for
+// 1.6 GB): a lane holds two neighbouring coordinates, loads them as one word where
+// rows start on 8 bytes and stores them as one of h and one of l, all loads of its
+// rows are issued before the first is used, and the registers leave room for four
+// CTAs an SM, or five (m = 1 million, d = 180: 310 us at 80 registers, 273 at 64; six
+// at 40 spill).  Short rows would leave most of a warp idle: with a warp a row
+// the self-join of 20000 points, d = 3, took 19 us here, with 8 lanes 9.
 template <int LANES, int NJ>
 __global__ void __launch_bounds__(256, LANES > 8 && NJ == 1 ? 5 : 4)
 prepare_pair_kernel(const float* __restrict__ R, int64_t m, int64_t tiles,
-                                    const float* __restrict__ centre, const float* __restrict__ Q,
-                                    int64_t n, int32_t d, int32_t kp,
-                                    uint32_t* __restrict__ R_lp, uint32_t* __restrict__ Q_lp,
-                                    float* __restrict__ qnorm, int64_t ref_warps,
-                                    int32_t* __restrict__ count0, int32_t* __restrict__ count1) {
+                    const float* __restrict__ centre, const float* __restrict__ Q, int64_t n,
+                    int32_t d, int32_t kp, uint32_t* __restrict__ R_lp, uint32_t* __restrict__ Q_lp,
+                    float* __restrict__ qnorm, int64_t ref_warps, int32_t* __restrict__ count0,
+                    int32_t* __restrict__ count1) {
     chain_begin();
     constexpr int RW = kPairRows, RPW = 32 / LANES;   // RPW rows side by side in a warp
     const int lane = threadIdx.x % LANES, grp = threadIdx.x % 32 / LANES;
