@@ -41,12 +41,12 @@ WORKLOAD = "uniform_n38400_d96_k20"
 SERVE_WORKLOAD = "serve_m4194304_d96"
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # DRAM traffic of one tensor-core filter launch on this workload, from one ncu
-# capture (dram__bytes_read.sum + dram__bytes_write.sum: 36.51 + 63.00 MB; see
+# capture (dram__bytes_read.sum + dram__bytes_write.sum: 33.75 + 62.75 MB; see
 # profiles/tc_filter_uniform_n38400_d96_k20.md), valid only for the kernel's
 # device source it was measured on (sha256 prefix of tc_device.cuh followed by
 # tc_ptx.cuh); otherwise reported as null.
-FILTER_TRAFFIC_BYTES = 99.23e6
-FILTER_TRAFFIC_SRC = "847a37a8c20ca9ba"
+FILTER_TRAFFIC_BYTES = 96.51e6
+FILTER_TRAFFIC_SRC = "e9255bd2387e75bd"
 FILTER_SOURCES = ("tc_device.cuh", "tc_ptx.cuh")
 
 CLOCK_HOLD_S = 0.3
@@ -498,7 +498,7 @@ def configs(args):
     w = inputs.WORKLOADS[SERVE_WORKLOAD]
     Rs = torch.from_numpy(inputs.workload_refs(SERVE_WORKLOAD)).to(dev)
     pool = torch.from_numpy(inputs.uniform(8192, w["d"], seed=w["seed_q"])).to(dev)
-    kp = (w["d"] + 4 + 63) // 64 * 64
+    kp = (w["d"] + 4 + 15) // 16 * 16    # rows end with a 32-byte MMA K step
     r_bytes = float(w["m"]) * kp * 2
     serve_rows = {}
     for b in (1, 64, 512, 4096):
@@ -550,7 +550,7 @@ def serve_batch(args):
         times.append(e0.elapsed_time(e1))
         filt.append(ix.profile().get("tc_filter", float("nan")))
     ix.close()
-    kp = (w["d"] + 4 + 63) // 64 * 64
+    kp = (w["d"] + 4 + 15) // 16 * 16    # rows end with a 32-byte MMA K step
     r_bytes = float(w["m"]) * kp * 2
     fms = float(np.median(filt))
     print(json.dumps({"serve_batch": b, "m": w["m"], "d": w["d"], "k": 20, "precision": "bf16",
