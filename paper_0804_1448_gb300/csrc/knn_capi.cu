@@ -375,8 +375,8 @@ struct SearchPlan {
 // small-set select's: one query among 5000 references, d = 8, 30 us against 97 us
 // with the CUDA-core select; 64 among 2 million, d = 96, 0.80 ms against 1.96; 4000
 // among 100000, d = 128, 0.44 ms against 3.90; n = m = 38400, d = 96, 0.86 ms
-// against 8.57.  Where the points are too dense for it (k = 10: from m = 5400 on
-// at d = 1, 550000 at d = 2, 40 million at d = 3) it would filter, certify next to
+// against 8.57.  Where the points are too dense for it (k = 10: from m = 5200 on
+// at d = 1, 510000 at d = 2, 36 million at d = 3) it would filter, certify next to
 // nothing and take the select all the same: n = 300, m = 4 million, d = 2, 3.1 ms
 // against 2.5, and n = 16 through the exact fallback 66 ms against 0.9.
 bool plan_pair(int64_t n, int64_t m, int32_t d, int32_t k, int sm_share, SearchPlan* p) {

@@ -219,13 +219,14 @@ bool pair_rows_fit(int32_t d) { return d >= 1 && d <= kPairMaxD; }
 // For points uniform in a cube of side 1, d / 12 from their centre on average
 // (squared), the slack is s = d / 12 (2 eq + 2 er + a), rows' remainders added, and
 // the k-th distance r^2 = (k / (m V_d))^(2 / d), V_d the volume of the unit ball, so
-// k ((1 + s / r^2)^(d / 2) - 1) = L references are expected in between.  3 L + 5
+// k ((1 + s / r^2)^(d / 2) - 1) = L references are expected in between.  3 L + 6
 // sqrt(L) + 4 covers the spread of their number and the corners of the cube,
-// whose rows lie further out, for all but a query in some ten thousand (with 2.5 L +
-// 4 sqrt(L) + 4, one of 4096 was left over at m = 100000, d = 2, k = 10: 247 us, 145
-// without it).  L is below 1 from d = 4 on, and large where the points are dense on
-// the scale of their spread: k = 10, 0.2 at d = 3, m = 100000, 2.5 at m = 4 million; 2.4
-// at d = 2, m = 100000, 24 at m = 1 million; 12 at d = 1, m = 5000.
+// whose rows lie further out, for all but a query in some ten thousand (simulated:
+// m = 100000, d = 2, L = 2.4, of 4096 queries a thousandth needed 14 to 17, the worst
+// one 19 to 22, and 21 are kept; m = 300000, L = 7.2, 38 at most, 42 kept).  L is
+// below 1 from d = 4 on, and large where the points are dense on the scale of
+// their spread: k = 10, 0.2 at d = 3, m = 100000, 2.5 at m = 4 million; 2.4 at d = 2, m =
+// 100000, 24 at m = 1 million; 12 at d = 1, m = 5000.
 int64_t pair_candidates(int64_t m, int32_t d, int32_t k) {
     constexpr double kPi = 3.14159265358979323846;
     const PairSlack ps = pair_slack(d);
@@ -234,7 +235,7 @@ int64_t pair_candidates(int64_t m, int32_t d, int32_t k) {
     const double log_v = 0.5 * d * std::log(kPi) - std::lgamma(0.5 * d + 1.0);
     const double r2 = std::exp(2.0 / d * (std::log(static_cast<double>(k) / static_cast<double>(m)) - log_v));
     const double l = k * std::expm1(0.5 * d * std::log1p(s / r2));
-    const double need = k + std::ceil(3.0 * l + 5.0 * std::sqrt(l) + 4.0);
+    const double need = k + std::ceil(3.0 * l + 6.0 * std::sqrt(l) + 4.0);
     return need <= static_cast<double>(m) ? static_cast<int64_t>(need) : m + 1;
 }
 
